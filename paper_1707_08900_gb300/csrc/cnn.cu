@@ -17,8 +17,9 @@
 //   chunk-major layout whose one-point frame holds the periodic copies, so a
 //   halo never wraps.  The input gradient is the same kernel with the
 //   weights transposed in channels and flipped in taps.
-// * The weight gradient sums over all grid points (K = points) on CUDA cores
-//   in FP32, split over CTAs and reduced in a fixed order (deterministic).
+// * The weight gradient sums over all grid points (K = points) on the tensor
+//   cores too (wgrad.cuh), split over CTAs and reduced in a fixed order
+//   (deterministic).
 // * MSE loss, Adam (FP32 master weights, BF16 copies in both GEMM layouts),
 //   input normalisation, the residual update of the solver state, and the
 //   centred box filter that makes training targets from fine-grid runs.
@@ -26,6 +27,7 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -521,100 +523,13 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
         tc::tmem_dealloc(tmem, SM::TCOLS);
 }
 
-// Weight (and bias) gradient of one layer, summed over this CTA's share of
-// the points: dW[co][tap][ci] += dY[p][co] X[p + tap][ci]; db[co] += dY[p][co].
-// dY and X are padded chunk-major activations (B samples allocated), so the
-// neighbour p + tap is read without any wrap arithmetic.
-template <int CO, int CI>
-__global__ void __launch_bounds__(TAPS *(CI / 4)) k_wgrad(const bf16 *__restrict__ dY,
-                                                          const bf16 *__restrict__ X, int n,
-                                                          int npts, int B, float *__restrict__ part)
-{
-    constexpr int NT = TAPS * (CI / 4);
-    __shared__ __align__(16) bf16 sdy[MT * CO];
-    const int t = threadIdx.x;
-    const int tap = t / (CI / 4), cq = t % (CI / 4);
-    const int dz = tap / 9 - 1, dyo = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-    const int n2 = n * n, n3 = n2 * n;
-    float acc[CO][4];
-    float db[CO];
-#pragma unroll
-    for (int c = 0; c < CO; ++c) {
-        db[c] = 0.f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            acc[c][i] = 0.f;
-    }
-    const long long chunk = ((long long)npts + gridDim.x - 1) / gridDim.x;
-    const long long p0 = chunk * blockIdx.x;
-    const long long p1 = min((long long)npts, p0 + chunk);
-    const uint4 *dY4 = reinterpret_cast<const uint4 *>(dY);
-    for (long long base = p0; base < p1; base += MT) {
-        const int cnt = (int)min((long long)MT, p1 - base);
-        __syncthreads();
-        for (int i = t; i < cnt * (CO / 8); i += NT) {
-            const int j = i / (CO / 8), c8 = i % (CO / 8);
-            const long long p = base + j;
-            const int b = (int)(p / n3);
-            int r = (int)(p - (long long)b * n3);
-            const int z = r / n2;
-            r -= z * n2;
-            reinterpret_cast<uint4 *>(sdy)[i] =
-                __ldg(dY4 + aidx(c8, b, z + 1, r / n + 1, r % n + 1, n, B));
-        }
-        __syncthreads();
-        for (int j = 0; j < cnt; ++j) {
-            const long long p = base + j;
-            const int b = (int)(p / n3);
-            int r = (int)(p - (long long)b * n3);
-            const int z = r / n2;
-            r -= z * n2;
-            const int y = r / n;
-            const int x = r - y * n;
-            const long long q =
-                aidx(cq / 2, b, z + 1 + dz, y + 1 + dyo, x + 1 + dx, n, B) * 8 + (cq % 2) * 4;
-            const uint2 xr = __ldg(reinterpret_cast<const uint2 *>(X + q));
-            const float2 x01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xr.x));
-            const float2 x23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xr.y));
-            const float xv[4] = {x01.x, x01.y, x23.x, x23.y};
-#pragma unroll
-            for (int c = 0; c < CO; c += 2) {
-                const float2 d = __bfloat1622float2(
-                    *reinterpret_cast<const __nv_bfloat162 *>(sdy + j * CO + c));
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    acc[c][i] += d.x * xv[i];
-                    acc[c + 1][i] += d.y * xv[i];
-                }
-                db[c] += d.x;
-                db[c + 1] += d.y;
-            }
-        }
-    }
-    float *out = part + (long long)blockIdx.x * (CO * TAPS * CI + CO);
-#pragma unroll
-    for (int c = 0; c < CO; ++c)
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            out[(c * TAPS + tap) * CI + 4 * cq + i] = acc[c][i];
-    if (t == 0)
-#pragma unroll
-        for (int c = 0; c < CO; ++c)
-            out[CO * TAPS * CI + c] = db[c];
-}
+}  // namespace cnn
+}  // namespace gbfd
 
-// g[i] = sum over CTAs of part[cta][i], fixed order.
-__global__ void k_reduce_parts(const float *__restrict__ part, int nparts, int count,
-                               float *__restrict__ g)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count)
-        return;
-    float s = 0.f;
-    for (int c = 0; c < nparts; ++c)
-        s += part[(long long)c * count + i];
-    g[i] = s;
-}
+#include "wgrad.cuh"
+
+namespace gbfd {
+namespace cnn {
 
 // Normalised BF16 input of layer 1 (C0 = 16 channels, zero beyond the nf
 // physical fields) at point (b, x, y, z) into the padded chunk-major x0,
@@ -858,6 +773,8 @@ struct gbfd_cnn {
     int grid_default;   // one per SM
     // TMA maps of the convolution inputs (padded chunk-major activations)
     CUtensorMap map_x0, map_a1, map_a2, map_dy3, map_dh2;
+    // and of the weight gradients' A (32 channels) and B operands
+    CUtensorMap wa_a2, wa_dh2, wa_dh1, wb_dy3, wb_a1, wb_x0;
     int64_t launches;
     char err[512];
 };
@@ -886,10 +803,9 @@ size_t al(size_t v) { return (v + 1023) & ~(size_t)1023; }
 struct CnnPlan {
     size_t off[32];
     size_t total;
-    int nparts;
 };
 
-constexpr int kWgradParts = 296;  // CTAs of the weight-gradient kernels
+constexpr int kWgradParts = 296;  // most CTAs of the weight-gradient kernels
 
 CnnPlan plan_for(int n, int batch)
 {
@@ -904,7 +820,7 @@ CnnPlan plan_for(int n, int batch)
         npad * C0 * 2, npad * CH * 2, npad * CH * 2, npad * C3 * 2, npad * CH * 2,
         npad * CH * 2,                                                    // bf16 acts
         np * CH * 4, np * CH * 4, np * 8 * 4,                             // h1 h2 y3
-        (size_t)kWgradParts * (CH * TAPS * CH + CH) * 4,                 // parts
+        (size_t)kWgradParts * wg::part_floats<true>() * 4,               // parts
         ((np + 255) / 256 + 8) * 8, 64, 256};
     size_t off = 0;
     const int cnt = sizeof(sizes) / sizeof(sizes[0]);
@@ -913,7 +829,6 @@ CnnPlan plan_for(int n, int batch)
         off = al(off + sizes[i]);
     }
     pl.total = off;
-    pl.nparts = kWgradParts;
     return pl;
 }
 
@@ -990,6 +905,35 @@ bool encode_act_map(CUtensorMap *m, const bf16 *base, int n, int B, int cin)
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// TMA maps of the weight gradients' operands (wgrad.cuh), boxes of one tile.
+// A, 32 channels: (8 interior x points, chunk, z with its frame, interior y,
+// sample).  B wide, 32 channels: (x, chunk, y with their frame, interior z,
+// sample).  B narrow, chunk 0 only: (interior x, x shift, y with its frame,
+// interior z, sample), the shift dimension one point (16 bytes) apart.
+// Outside a map's extents the copy fills zeros.
+enum { WG_A, WG_B_WIDE, WG_B_NARROW };
+bool encode_wgrad_map(CUtensorMap *m, const bf16 *base, int n, int B, int kind)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
+    if (!fn)
+        return false;
+    const cuuint64_t N = (cuuint64_t)n, P = N + 2, row = P * 16, plane = P * row, vol = P * plane;
+    const cuuint64_t chunk = vol * (cuuint64_t)B, nb = (cuuint64_t)B;
+    const char *p = reinterpret_cast<const char *>(base) + (kind == WG_A ? row + 16 : plane);
+    const cuuint64_t dims[3][5] = {
+        {8 * N, 4, P, N, nb}, {8 * P, 4, P, N, nb}, {8 * N, 3, P, N, nb}};
+    const cuuint64_t strides[3][4] = {
+        {chunk, plane, row, vol}, {chunk, row, plane, vol}, {16, row, plane, vol}};
+    const cuuint32_t box[3][5] = {{8 * wg::TX, 4, wg::AZ, wg::TY, 1},
+                                  {8 * (wg::TX + 2), 4, wg::BY, wg::ZB, 1},
+                                  {8 * wg::TX, 3, wg::BY, wg::ZB, 1}};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<char *>(p), dims[kind],
+              strides[kind], box[kind], estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 cudaError_t pack(gbfd_cnn *c, const float *g, float lr)
 {
     PackArgs a;
@@ -1045,16 +989,32 @@ cudaError_t forward(gbfd_cnn *c, int npts, bool keep)
     return conv<CH, C3, EPI_LINEAR>(c, c->map_a2, a);
 }
 
-template <int CO, int CI>
-cudaError_t wgrad(gbfd_cnn *c, const bf16 *dY, const bf16 *X, int npts, float *g)
+// Weight and bias gradients of one layer: A and B are the staged operands of
+// wgrad.cuh (SWAP: A = X, B = dY), one CTA per SM (fewer on request).
+template <int CO, int CI, bool WIDE, bool SWAP>
+cudaError_t wgrad(gbfd_cnn *c, const CUtensorMap &amap, const CUtensorMap &bmap, int npts, float *g)
 {
-    k_wgrad<CO, CI><<<c->nparts, TAPS * (CI / 4), 0, c->stream>>>(dY, X, c->n, npts, c->batch,
-                                                                    c->parts);
-    cudaError_t e = cudaGetLastError();
+    auto k = wg::k_wgrad_tc<WIDE>;
+    constexpr int smem = wg::Smem<WIDE>::BYTES;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess)
         return e;
-    const int count = CO * TAPS * CI + CO;
-    k_reduce_parts<<<(count + 255) / 256, 256, 0, c->stream>>>(c->parts, c->nparts, count, g);
+    const int n = c->n;
+    wg::Args a;
+    a.n = n;
+    a.nb = (int)(npts / ((long long)n * n * n));
+    a.bias_b = SWAP;
+    a.part = c->parts;
+    a.dev_error = c->derr;
+    const long long ntiles = (long long)a.nb * ((n + wg::ZB - 1) / wg::ZB) *
+                             ((n + wg::TY - 1) / wg::TY) * ((n + wg::TX - 1) / wg::TX);
+    const int grid = (int)std::min<long long>(ntiles, c->nparts);
+    k<<<grid, wg::THREADS, smem, c->stream>>>(amap, bmap, a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess)
+        return e;
+    wg::k_wgrad_reduce<CO, CI, WIDE, SWAP>
+        <<<(wg::part_floats<WIDE>() + 31) / 32, 256, 0, c->stream>>>(c->parts, grid, g);
     c->launches += 2;
     return cudaGetLastError();
 }
@@ -1073,7 +1033,7 @@ cudaError_t backward(gbfd_cnn *c, const float *xs, const float *ts, int nf, int 
     if (e != cudaSuccess)
         return e;
     // layer 3: weight gradient, then input gradient through GELU'(h2)
-    e = wgrad<C3, CH>(c, c->dy3, c->a2, npts, c->g + poff(2));
+    e = wgrad<C3, CH, false, true>(c, c->wa_a2, c->wb_dy3, npts, c->g + poff(2));
     if (e != cudaSuccess)
         return e;
     ConvArgs a;
@@ -1089,7 +1049,7 @@ cudaError_t backward(gbfd_cnn *c, const float *xs, const float *ts, int nf, int 
     if (e != cudaSuccess)
         return e;
     // layer 2
-    e = wgrad<CH, CH>(c, c->dh2, c->a1, npts, c->g + poff(1));
+    e = wgrad<CH, CH, true, false>(c, c->wa_dh2, c->wb_a1, npts, c->g + poff(1));
     if (e != cudaSuccess)
         return e;
     a.wB = c->bwd[1];
@@ -1099,7 +1059,7 @@ cudaError_t backward(gbfd_cnn *c, const float *xs, const float *ts, int nf, int 
     if (e != cudaSuccess)
         return e;
     // layer 1: weight gradient only
-    return wgrad<CH, C0>(c, c->dh1, c->x0, npts, c->g + poff(0));
+    return wgrad<CH, C0, false, false>(c, c->wa_dh1, c->wb_x0, npts, c->g + poff(0));
 }
 
 gbfd_status check(gbfd_cnn *c, int batch)
@@ -1179,7 +1139,6 @@ gbfd_status gbfd_cnn_init(int n, int batch, void *workspace, size_t workspace_by
     c->lparts = (double *)(b + pl.off[k++]);
     c->loss = (double *)(b + pl.off[k++]);
     c->derr = (int *)(b + pl.off[k++]);
-    c->nparts = pl.nparts;
     c->adam_t = 0;
     c->launches = 0;
     c->err[0] = 0;
@@ -1188,12 +1147,19 @@ gbfd_status gbfd_cnn_init(int n, int batch, void *workspace, size_t workspace_by
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     c->grid_conv = c->grid_default = sms > 0 ? sms : 1;
+    c->nparts = std::min(c->grid_default, kWgradParts);
     if (e == cudaSuccess &&
         !(encode_act_map(&c->map_x0, c->x0, n, batch, C0) &&
           encode_act_map(&c->map_a1, c->a1, n, batch, CH) &&
           encode_act_map(&c->map_a2, c->a2, n, batch, CH) &&
           encode_act_map(&c->map_dy3, c->dy3, n, batch, C3) &&
-          encode_act_map(&c->map_dh2, c->dh2, n, batch, CH))) {
+          encode_act_map(&c->map_dh2, c->dh2, n, batch, CH) &&
+          encode_wgrad_map(&c->wa_a2, c->a2, n, batch, WG_A) &&
+          encode_wgrad_map(&c->wa_dh2, c->dh2, n, batch, WG_A) &&
+          encode_wgrad_map(&c->wa_dh1, c->dh1, n, batch, WG_A) &&
+          encode_wgrad_map(&c->wb_dy3, c->dy3, n, batch, WG_B_NARROW) &&
+          encode_wgrad_map(&c->wb_a1, c->a1, n, batch, WG_B_WIDE) &&
+          encode_wgrad_map(&c->wb_x0, c->x0, n, batch, WG_B_NARROW))) {
         cerr(nullptr, "cnn init: TMA descriptor encoding failed");
         delete c;
         return GBFD_ERR_CUDA;
@@ -1236,7 +1202,7 @@ gbfd_status gbfd_cnn_set_option(gbfd_cnn *c, int key, int64_t value)
     case GBFD_CNN_OPT_WGRAD_PARTS:
         if (value < 0 || value > kWgradParts)
             break;
-        c->nparts = value == 0 ? kWgradParts : (int)value;
+        c->nparts = value == 0 ? std::min(c->grid_default, kWgradParts) : (int)value;
         return GBFD_OK;
     default:
         break;

@@ -45,6 +45,11 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
            | ((uint32_t)(M >> 4) << 24);   // M / 16
 }
 
+// Instruction descriptor bits that make A / B MN-major (M or N contiguous in
+// each core matrix: 8 K rows of 16 bytes); the operand's descriptor then takes
+// the K-group stride as LBO and the stride between 8-wide M or N chunks as SBO.
+constexpr uint32_t kIdescTransA = 1u << 15, kIdescTransB = 1u << 16;
+
 // D(tmem) (+)= A(smem) * B(smem)^T, issued by one thread.
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                          uint32_t idesc, uint32_t accumulate)
