@@ -38,7 +38,7 @@ struct gbfd_ctx {
     int64_t launches;
     int kernel_path;  // 0 = tiled when supported, 1 = simple
     int tile_cfg;     // index into the tiled kernel's tile table (-1 = default)
-    int sms;          // SM count of the context's device (read at init)
+    int zc;           // planes per CTA of the default tiled kernel (default_zc)
     double h[3];      // grid spacings (z: lz / (nz - 1) between walls)
     int fault_skip;   // test-only fault injection (-1 = off)
     int host_path;    // 0 = pinned host buffers accessed in place, 1 = always staged
@@ -200,6 +200,7 @@ StateBufs bufs(gbfd_ctx *c)
     b.div = c->div_region ? c->div_region + c->Ld.origin : nullptr;
     b.Ls = c->Ls;
     b.Lw = c->Lw;
+    b.zc = c->zc;
     return b;
 }
 
@@ -268,31 +269,6 @@ bool write_cache(const char *path, const std::map<std::string, std::pair<int, do
     return rename(tmp.c_str(), path) == 0;
 }
 
-// The FP32 default's z-chunk length for this grid (S = resident CTAs of the
-// default kernel: 32 x 8 tiles, two per SM): 64 planes when that makes at
-// least 16 launch waves (512^3: 27 waves, 3% faster than 40 there, the halo
-// planes falling from 15% to 9%); else 40 when that still makes at least
-// four waves (fewest halo planes, and 7 chunks of a 256 column fill 5.9
-// waves where 8 chunks of 32 fill 6.7); else 32 when that fills at least
-// half a wave; else 16 when that fills a quarter; else 8, so that small grids
-// (64^3: 128 CTAs of 8 planes) keep more SMs busy and each CTA's plane
-// pipeline short.  Measured best at 128^3 (32), 256^3 (40) and 512^3 (64).
-int fp32_default_cfg(const gbfd_ctx *c)
-{
-    const long long slots = 2LL * c->sms;
-    const long long tiles = (long long)((c->p.nx + 31) / 32) * ((c->p.ny + 7) / 8);
-    // positions of 40, 32, 64, 16 and 8 in the tile table's chunk list
-    if (tiles * ((c->p.nz + 63) / 64) >= 16 * slots)
-        return kDefaultF32 + 2;
-    if (tiles * ((c->p.nz + 39) / 40) >= 4 * slots)
-        return kDefaultF32;
-    if (2 * tiles * ((c->p.nz + 31) / 32) >= slots)
-        return kDefaultF32 + 1;
-    if (4 * tiles * ((c->p.nz + 15) / 16) >= slots)
-        return kDefaultF32 + 3;
-    return kDefaultF32 + 4;
-}
-
 gbfd_status do_substep(gbfd_ctx *c, int s, double dt)
 {
     StateBufs b = bufs(c);
@@ -313,8 +289,7 @@ gbfd_status do_substep(gbfd_ctx *c, int s, double dt)
     case GBFD_FP32:
         e = tiled ? launch_substep_tiled<float, float, float>(
                         b, c->c32, st, c->nf, c->p.form,
-                        c->tile_cfg < 0 ? fp32_default_cfg(c) : c->tile_cfg, c->dev_error,
-                        &c->tmaps, c->stream, &n)
+                        c->tile_cfg, c->dev_error, &c->tmaps, c->stream, &n)
                   : launch_substep_simple<float, float, float>(b, c->c32, st, c->nf, c->p.form,
                                                                c->stream, &n);
         break;
@@ -327,10 +302,8 @@ gbfd_status do_substep(gbfd_ctx *c, int s, double dt)
         break;
     case GBFD_FP32_ACCFF:
         e = tiled ? launch_substep_tiled<float, float, ffloat>(b, c->c32, st, c->nf, c->p.form,
-                                                               c->tile_cfg < 0 ? fp32_default_cfg(c)
-                                                                               : c->tile_cfg,
-                                                               c->dev_error, &c->tmaps, c->stream,
-                                                               &n)
+                                                               c->tile_cfg, c->dev_error, &c->tmaps,
+                                                               c->stream, &n)
                   : launch_substep_simple<float, float, ffloat>(b, c->c32, st, c->nf, c->p.form,
                                                                 c->stream, &n);
         break;
@@ -450,14 +423,17 @@ gbfd_status gbfd_init(const gbfd_params *p, void *workspace, size_t workspace_by
     c->tile_cfg = -1;
     {
         // the device current at init is the context's device
-        int dev = 0;
-        c->sms = 0;
+        int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            c->sms <= 0) {
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            sms <= 0) {
             (void)cudaGetLastError();
-            c->sms = 152;
+            sms = 152;
         }
+        // xy tiles of the default kernels: 32 x 8 (FP32 storage), 16 x 8 (FP64)
+        const int tx = c->sbytes == 8 ? 16 : 32;
+        c->zc = default_zc(c->sbytes, (long long)((p->nx + tx - 1) / tx) * ((p->ny + 7) / 8), p->nz,
+                           sms);
     }
     c->fault_skip = -1;
     c->host_path = 0;

@@ -407,6 +407,7 @@ struct StateBufs {
     void *div;   // padded divergence field (19-point form)
     Layout Ls;   // layout of in/out/div (div uses one field)
     Layout Lw;   // layout of w
+    int zc;      // planes per CTA of the default tiled kernel on this grid
 };
 
 }  // namespace gbfd

@@ -61,6 +61,11 @@ constexpr int kDefaultF64 = 5 * kZcChoices;
 int tiled_config_count(int sbytes);
 TileConfig tiled_config(int sbytes, int i);
 
+// Planes per CTA of the default kernels on a grid of `tiles` xy tiles and nz
+// planes (w = 4: FP32 storage, 8: FP64 storage), from a model of the launch
+// that reproduces the measured optimum to about 1% (tiled_common.cu).
+int default_zc(int w, long long tiles, int nz, int sms);
+
 // Encoded TMA descriptors of the state buffers, cached per context.
 struct TmapCache {
     static constexpr int kEntries = 16;

@@ -3,8 +3,8 @@
 // kernel, the two-plane packed two-point kernel, and the kernel that
 // finishes output planes three planes behind the in-plane work (pending
 // right-hand sides in registers, two or one steps per iteration, or in TMEM:
-// the default; its warp-shuffle variant is compiled in tiled_shfl.cu).  The z-chunk length comes from the table entry; the API picks
-// the default entry's chunk per grid (fp32_default_cfg in api.cu).
+// the default; its warp-shuffle variant is compiled in tiled_shfl.cu).  The z-chunk length comes from the table entry, the
+// default's from the grid (default_zc).
 #include "tiled4_impl.cuh"
 
 namespace gbfd {
@@ -15,7 +15,9 @@ cudaError_t launch_substep_tiled(const StateBufs &b, const Coef<TS> &c, const RK
                                  cudaStream_t stream, int *launches)
 {
     const int idx = cfg < 0 ? kDefaultF32 : cfg;
-    const TileConfig t = tiled_config(4, idx);
+    TileConfig t = tiled_config(4, idx);
+    if (cfg < 0)
+        t.zc = b.zc;
     // a forced step (Sect. 6 forcing) runs on the default kernel, whatever
     // the tile table entry
     const int v = st.fo.on ? kDefaultF32 / kZcChoices : idx / kZcChoices;

@@ -15,7 +15,9 @@ cudaError_t launch_substep_tiled(const StateBufs &b, const Coef<TS> &c, const RK
     if (form != 0)
         return cudaErrorNotSupported;
     const int idx = cfg < 0 ? kDefaultF32 : cfg;
-    const TileConfig t = tiled_config(4, idx);
+    TileConfig t = tiled_config(4, idx);
+    if (cfg < 0)
+        t.zc = b.zc;
     return launch_lag_cfg<TW, TA, 32, 8, 8, 2, true>(b, c, st, nf, t.zc, kVarLagTm, dev_error, cache,
                                                    stream, launches);
 }
