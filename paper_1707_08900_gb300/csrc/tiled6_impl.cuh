@@ -17,8 +17,14 @@
 //     13.4 KB (16 x 8 tile, 3-cell halo, 5 fields), three CTAs per SM where
 //     the 7-plane ring of the one-point kernel allows two.  u-tilde comes
 //     from global memory, loaded at the start of the step that uses it.
+//   * folded weights (FoldCoef, common.cuh): the viscosity, the time step and
+//     the signs are in the stencil weights, so every derivative goes straight
+//     into the right-hand side: 245 FP64 operations per point and substep
+//     where separate Laplacian, divergence, advection and update products
+//     take 285.
 // Output plane o waits three planes for its z-paired terms; the rest of its
-// right-hand side waits in tensor memory (4 slots, 2 columns per FP64 value).
+// right-hand side (times dt) waits in tensor memory (4 slots, 2 columns per
+// FP64 value).
 #pragma once
 
 #include "tcgen05.cuh"
@@ -131,7 +137,7 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
     const bool valid = (x < Ls.nx) && (y < Ls.ny);
     const int toff = (ty + GY) * BX + (tx + GX);
     const bool first = st.first != 0, last = st.last != 0;
-    const double alpha = st.alpha, beta = st.beta, dt = st.dt;
+    const double alpha = st.alpha, beta = st.beta;
     const int skip_plane = blockIdx.x == 0 && blockIdx.y == 0 ? skip_plane_arg : -1;
 
     int issued = 0;
@@ -172,12 +178,12 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
         acx[m] = acy[m] = acz[m] = 0.0;
 
     // add the differences d[k-1] of one plane (accumulator index MC) with
-    // weights MX(pair, k): plus to the outputs below it, minus to those above
+    // weights M3(pair, k): plus to the outputs below it, minus to those above
     auto spread = [&](double *ac, const double *d, int pair, auto mcc) {
         constexpr int MC = decltype(mcc)::value;
 #pragma unroll
         for (int k = 1; k <= 3; ++k) {
-            const double mk = c.MX(pair, k);
+            const double mk = c.M3(pair, k);
             if (MC - k >= 0)
                 ac[MC - k] = fma(mk, d[k - 1], ac[MC - k]);
             if (MC + k < W)
@@ -266,11 +272,15 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
         auto ld = [&](int f, int dy, int dx) -> double {
             return sm[cb + f * FSTRIDE + dy * BX + dx];
         };
-        double g[3], d2[3], hx[3], hy[3];
-        // Eqs. 6-7 along x, y, z for field f; hx, hy keep the differences
-        auto axial = [&](int f, bool second) {
-            const double cc = colv[f][3];
-            double ax, ay, az, bx, by, bz;
+        double g[3], hx[3], hy[3];
+        // Eqs. 6-7 along x, y, z for field f: the gradient (L: grad lnrho,
+        // else -dt grad) into g, the weighted second derivatives of velocity
+        // component I >= 0 onto acc; hx, hy keep the differences
+        auto axial = [&](int f, auto lc, auto ic, double &acc) {
+            constexpr bool L = decltype(lc)::value;
+            constexpr int I = decltype(ic)::value;
+            auto w1 = [&](int a, int k) { return L ? c.L1(a, k) : c.N1(a, k); };
+            auto w2 = [&](int a, int k) { return a == I ? c.X2(a, k) : c.V2(a, k); };
 #pragma unroll
             for (int k = 1; k <= 3; ++k) {
                 const double xp = ld(f, 0, k), xm = ld(f, 0, -k);
@@ -279,109 +289,76 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
                 hx[k - 1] = xp - xm;
                 hy[k - 1] = yp - ym;
                 const double dz = zp - zm;
-                if (k == 1) {
-                    ax = c.D1(0, 1) * hx[0];
-                    ay = c.D1(1, 1) * hy[0];
-                    az = c.D1(2, 1) * dz;
-                } else {
-                    ax = fma(c.D1(0, k), hx[k - 1], ax);
-                    ay = fma(c.D1(1, k), hy[k - 1], ay);
-                    az = fma(c.D1(2, k), dz, az);
+                g[0] = k == 1 ? w1(0, 1) * hx[0] : fma(w1(0, k), hx[k - 1], g[0]);
+                g[1] = k == 1 ? w1(1, 1) * hy[0] : fma(w1(1, k), hy[k - 1], g[1]);
+                g[2] = k == 1 ? w1(2, 1) * dz : fma(w1(2, k), dz, g[2]);
+                if constexpr (I >= 0) {
+                    acc = fma(w2(0, k), xp + xm, acc);
+                    acc = fma(w2(1, k), yp + ym, acc);
+                    acc = fma(w2(2, k), zp + zm, acc);
                 }
-                if (second) {
-                    if (k == 1) {
-                        bx = c.D2c(0) * cc;
-                        by = c.D2c(1) * cc;
-                        bz = c.D2c(2) * cc;
-                    }
-                    bx = fma(c.D2(0, k), xp + xm, bx);
-                    by = fma(c.D2(1, k), yp + ym, by);
-                    bz = fma(c.D2(2, k), zp + zm, bz);
-                }
-            }
-            g[0] = ax;
-            g[1] = ay;
-            g[2] = az;
-            if (second) {
-                d2[0] = bx;
-                d2[1] = by;
-                d2[2] = bz;
             }
         };
-        // Eq. 8 in the (x, y) plane
-        auto mix_xy = [&](int f) -> double {
-            double a;
+        // Eq. 8 in the (x, y) plane, onto acc
+        auto mix_xy = [&](int f, double &acc) {
 #pragma unroll
-            for (int k = 1; k <= 3; ++k) {
-                const double d = (ld(f, k, k) - ld(f, k, -k)) - (ld(f, -k, k) - ld(f, -k, -k));
-                a = k == 1 ? c.MX(0, 1) * d : fma(c.MX(0, k), d, a);
-            }
-            return a;
+            for (int k = 1; k <= 3; ++k)
+                acc = fma(c.M3(0, k), (ld(f, k, k) - ld(f, k, -k)) - (ld(f, -k, k) - ld(f, -k, -k)),
+                          acc);
         };
-        const double NU = c.nu, NU3 = c.nu3;
+        using NoComp = std::integral_constant<int, -1>;
         const double uc[3] = {colv[1][3], colv[2][3], colv[3][3]};
-        double acc[4], gl[3];
-        double dv = 0.0;
-        axial(0, false);
-        gl[0] = g[0];
-        gl[1] = g[1];
-        gl[2] = g[2];
+        double acc[3], gl[3], nng[3], q[3], dvm = 0.0;
+        axial(0, std::true_type{}, NoComp{}, acc[0]);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            axial(1 + i, true);
+        for (int a = 0; a < 3; ++a) {
+            gl[a] = g[a];
+            nng[a] = c.nnu * g[a];
+            q[a] = fma(c.nnu, g[a], uc[a]);
+        }
+        auto component = [&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            acc[i] = i == 0 ? c.VC(0) * uc[0] : fma(c.VC(i), uc[i], acc[i]);
+            axial(1 + i, std::false_type{}, ic, acc[i]);
             // this plane's differences: D_xz u_x and D_yz u_y -> z component,
             // D_xz u_z -> x, D_yz u_z -> y
-            if (i == 0) {
+            if constexpr (i == 0) {
                 spread(acz, hx, 1, MC3{});
-            } else if (i == 1) {
+            } else if constexpr (i == 1) {
                 spread(acz, hy, 2, MC3{});
             } else {
                 spread(acx, hx, 1, MC3{});
                 spread(acy, hy, 2, MC3{});
             }
-            double adv = uc[0] * g[0];
-            adv = fma(uc[1], g[1], adv);
-            adv = fma(uc[2], g[2], adv);
-            const double lap = d2[0] + d2[1] + d2[2];
-            double sg = g[0] * gl[0];
-            sg = fma(g[1], gl[1], sg);
-            sg = fma(g[2], gl[2], sg);
-            double ai = NU * (lap + sg);
-            if (i > 0)
-                ai += acc[1 + i];
-            ai -= adv;
-            ai = fma(NU3, d2[i], ai);
-            acc[1 + i] = ai;
-            // the d_a u_i d_i lnrho half of 2 S.grad lnrho, for every component a
-            const double nugl = NU * gl[i];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                if (a > i && i == 0)
-                    acc[1 + a] = g[a] * nugl;  // first contribution
-                else
-                    acc[1 + a] = fma(g[a], nugl, acc[1 + a]);
-            }
-            dv += g[i];
-            if (i == 0)
-                acc[2] = fma(NU3, mix_xy(1), acc[2]);  // D_xy u_x -> y
-            else if (i == 1)
-                acc[1] = fma(NU3, mix_xy(2), acc[1]);  // D_xy u_y -> x
-        }
-        if constexpr (NF == 5) {
-            axial(4, false);
-            double t = uc[0] * g[0];
-            t = fma(uc[1], g[1], t);
-            t = fma(uc[2], g[2], t);
-            prn[4] = -t;
-        }
+            for (int a = 0; a < 3; ++a)  // advection and d_a u_i d_a lnrho
+                acc[i] = fma(g[a], q[a], acc[i]);
+#pragma unroll
+            for (int a = 0; a < 3; ++a)  // d_a u_i d_i lnrho, for component a
+                acc[a] = i == 0 && a > 0 ? g[a] * nng[0] : fma(g[a], nng[i], acc[a]);
+            dvm = i == 0 ? g[0] : dvm + g[i];
+            if constexpr (i == 0)
+                mix_xy(1, acc[1]);  // D_xy u_x -> y
+            else if constexpr (i == 1)
+                mix_xy(2, acc[0]);  // D_xy u_y -> x
+        };
+        component(std::integral_constant<int, 0>{});
+        component(std::integral_constant<int, 1>{});
+        component(std::integral_constant<int, 2>{});
         double ug = uc[0] * gl[0];
         ug = fma(uc[1], gl[1], ug);
         ug = fma(uc[2], gl[2], ug);
-        prn[0] = -(ug + dv);
-        const double t = -c.nu23 * dv;
+        prn[0] = fma(c.ns, ug, dvm);
+        const double t = fma(c.nu23, dvm, c.ncs2);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-            prn[1 + a] = fma(t, gl[a], fma(-c.cs2, gl[a], acc[1 + a]));
+            prn[1 + a] = fma(t, gl[a], acc[a]);
+        if constexpr (NF == 5) {
+            axial(4, std::false_type{}, NoComp{}, acc[0]);
+            double r = uc[0] * g[0];
+            r = fma(uc[1], g[1], r);
+            prn[4] = fma(uc[2], g[2], r);
+        }
     };
 
     // u-tilde of the next output plane to finish (before the work that hides
@@ -398,17 +375,17 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
         }
     };
     // output plane o (accumulator and window index I): add the z-paired
-    // terms, apply Eq. 10, store the state (and ghost copies) and u-tilde
+    // terms, apply Eq. 10 (dt is in the weights), store the state (and ghost copies) and u-tilde
     auto finish = [&](const int o, auto ic, const double *wv) {
         constexpr int I = decltype(ic)::value;
         double r[NF];
         tm_get<NF>(trow + (uint32_t)((o & 3) * kTmSlotCols), r);
-        r[1] = fma(c.nu3, acx[I], r[1]);
-        r[2] = fma(c.nu3, acy[I], r[2]);
-        r[3] = fma(c.nu3, acz[I], r[3]);
+        r[1] += acx[I];
+        r[2] += acy[I];
+        r[3] += acz[I];
         if (valid) {
             if constexpr (FORCE) {
-                // f_i = amp_i cos(k.x + phi) (Sect. 6, Eqs. 20-21)
+                // f_i = amp_i cos(k.x + phi) (Sect. 6, Eqs. 20-21; amp times dt)
                 const double fc = forcing_cos<double>(st.fo, x, y, z0 + o);
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
@@ -416,7 +393,7 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
             }
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
-                const double wn = first ? dt * r[f] : fma(alpha, wv[f], dt * r[f]);
+                const double wn = first ? r[f] : fma(alpha, wv[f], r[f]);
                 const double ov = fma(beta, wn, colv[f][I]);
                 if (!last)
                     w[f * Lw.fpitch + go_w] = wn;
@@ -540,7 +517,10 @@ cudaError_t launch_lag64_cfg(const StateBufs &b, const Coef<double> &c, const RK
     const int skip_plane = st.fault_skip_plane;
     cudaError_t e;
     const bool iso = coef_is_cubic(c);
-    const CubicCoef<double> cc = cubic_of(c);
+    const FoldCoef<double> fc = make_fold<double>(c, st.dt);
+    RKStage sd = st;  // the forcing takes the time step too
+    for (int a = 0; a < 3; ++a)
+        sd.fo.amp[a] *= st.dt;
 #define GBFD_LAUNCH_L64_F(NFV, FRC, CT, CV)                                                       \
     do {                                                                                          \
         auto kern = tiled6::k_substep_lag64<NFV, TX, TY, NS, MINB, FRC, CT>;                      \
@@ -551,7 +531,7 @@ cudaError_t launch_lag64_cfg(const StateBufs &b, const Coef<double> &c, const RK
                                      (int)cudaSharedmemCarveoutMaxShared);                        \
         if (e != cudaSuccess)                                                                     \
             return e;                                                                             \
-        kern<<<grid, block, sm, stream>>>(*map, out, w, b.Ls, b.Lw, CV, st, zc, tiles_x,          \
+        kern<<<grid, block, sm, stream>>>(*map, out, w, b.Ls, b.Lw, CV, sd, zc, tiles_x,          \
                                           dev_error, skip_plane);                                 \
     } while (0)
 #define GBFD_LAUNCH_L64(NFV, CT, CV)                                                              \
@@ -563,14 +543,14 @@ cudaError_t launch_lag64_cfg(const StateBufs &b, const Coef<double> &c, const RK
     } while (0)
     if (nf == 5) {
         if (iso)
-            GBFD_LAUNCH_L64(5, CubicCoef<double>, cc);
+            GBFD_LAUNCH_L64(5, FoldCubic<double>, cubic_of(fc));
         else
-            GBFD_LAUNCH_L64(5, Coef<double>, c);
+            GBFD_LAUNCH_L64(5, FoldCoef<double>, fc);
     } else {
         if (iso)
-            GBFD_LAUNCH_L64(4, CubicCoef<double>, cc);
+            GBFD_LAUNCH_L64(4, FoldCubic<double>, cubic_of(fc));
         else
-            GBFD_LAUNCH_L64(4, Coef<double>, c);
+            GBFD_LAUNCH_L64(4, FoldCoef<double>, fc);
     }
 #undef GBFD_LAUNCH_L64
 #undef GBFD_LAUNCH_L64_F
