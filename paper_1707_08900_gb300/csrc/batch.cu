@@ -61,6 +61,12 @@ struct BoxDesc {
     int nitems;                  // columns of this box in the work list
 };
 
+// What a step's time steps make of each box, refreshed before every replay.
+struct BoxStep {
+    float dt;
+    FoldCubic<float> fold;  // the lagged routine's weights, dt folded in
+};
+
 // Device-side state of the dataflow launch, zeroed before each launch.
 struct Flow {
     int next;   // next work item to hand out
@@ -85,7 +91,7 @@ constexpr int smem_bytes()
 template <int KIND, int NF, bool SPEC = false>
 __device__ __forceinline__ bool run_item(const BoxDesc *__restrict__ B, const int4 item,
                                          const int s, const int parity, const float dt,
-                                         const int zc, const CubicCoef<float> &scoef, int &jrun,
+                                         const int zc, const FoldCubic<float> &scoef, int &jrun,
                                          int &wrun, unsigned char *smem, int *dev_error,
                                          const uint32_t tmem)
 {
@@ -98,6 +104,23 @@ __device__ __forceinline__ bool run_item(const BoxDesc *__restrict__ B, const in
     const float beta = s == 0 ? (float)(1.0 / 3.0) : (s == 1 ? (float)(15.0 / 16.0)
                                                             : (float)(8.0 / 15.0));
     if constexpr (KIND == KIND_LAG) {
+        if constexpr (SPEC && NF == 5) {
+            if (L.nx % TX == 0 && L.ny % TY == 0) {
+                auto run = [&](auto stg) {
+                    constexpr int S = decltype(stg)::value;
+                    return tiled4::run_column<float, float, NF, TX, TY, NS, U, false, false, true,
+                                              FoldCubic<float>, false, S, true>(
+                        &B->tm_state[wi][parity], &B->tm_w[wi], B->state[parity ^ 1], B->w, L, L,
+                        scoef, alpha, beta, dt, S == 0, S == 2, item.y, item.z, item.w, nout, jrun,
+                        wrun, smem, dev_error, -1, nullptr, tmem);
+                };
+                if (s == 0)
+                    return run(std::integral_constant<int, 0>{});
+                if (s == 1)
+                    return run(std::integral_constant<int, 1>{});
+                return run(std::integral_constant<int, 2>{});
+            }
+        }
         return tiled4::run_column<float, float, NF, TX, TY, NS, U, false, false, true>(
             &B->tm_state[wi][parity], &B->tm_w[wi], B->state[parity ^ 1], B->w, L, L, scoef,
             alpha, beta, dt, s == 0, s == 2, item.y, item.z, item.w, nout, jrun, wrun, smem,
@@ -158,12 +181,12 @@ __device__ __forceinline__ void tmem_close(uint32_t tmem)
 template <int KIND, int NF>
 __global__ void __launch_bounds__((kind_tx(KIND) / 2) * TY) k_batch_substep(
     const BoxDesc *__restrict__ boxes, const int4 *__restrict__ items, const int nitems,
-    const float *__restrict__ dts, const int zc, const int s, const int parity,
+    const BoxStep *__restrict__ steps, const int zc, const int s, const int parity,
     int *__restrict__ dev_error)
 {
     constexpr int SMB = smem_bytes<KIND, NF>();
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ CubicCoef<float> scoef;
+    __shared__ FoldCubic<float> scoef;
     if constexpr (KIND == KIND_LAG)
         tiled2::init_barriers(reinterpret_cast<uint64_t *>(
                                   smem + tiled4::RingL<float, NF, 32, TY, NS, U>::BAR_OFF),
@@ -181,9 +204,9 @@ __global__ void __launch_bounds__((kind_tx(KIND) / 2) * TY) k_batch_substep(
         const BoxDesc *B = boxes + item.x;
         __syncthreads();  // every thread is done with the previous box's weights
         if (threadIdx.x == 0)
-            scoef = B->coef;
+            scoef = steps[item.x].fold;
         __syncthreads();
-        if (!run_item<KIND, NF>(B, item, s, parity, dts[item.x], zc, scoef, jrun, wrun, smem,
+        if (!run_item<KIND, NF>(B, item, s, parity, steps[item.x].dt, zc, scoef, jrun, wrun, smem,
                                 dev_error, tmem))
             break;
     }
@@ -204,12 +227,12 @@ __device__ __forceinline__ int ld_acquire(const int *p)
 template <int KIND, int NF>
 __global__ void __launch_bounds__((kind_tx(KIND) / 2) * TY) k_batch_flow(
     const BoxDesc *__restrict__ boxes, const int4 *__restrict__ items, const int nitems,
-    const int nsub, const float *__restrict__ dts, const int zc, const int cur,
+    const int nsub, const BoxStep *__restrict__ steps, const int zc, const int cur,
     Flow *__restrict__ flow, int *__restrict__ dev_error, const int stall_item)
 {
     constexpr int SMB = smem_bytes<KIND, NF>();
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ CubicCoef<float> scoef;
+    __shared__ FoldCubic<float> scoef;
     __shared__ int sq;
     if constexpr (KIND == KIND_LAG)
         tiled2::init_barriers(reinterpret_cast<uint64_t *>(
@@ -256,7 +279,7 @@ __global__ void __launch_bounds__((kind_tx(KIND) / 2) * TY) k_batch_flow(
             }
             sq = q;
             if (q >= 0)
-                scoef = boxes[items[q % nitems].x].coef;
+                scoef = steps[items[q % nitems].x].fold;
         }
         __syncthreads();
         const int q = sq;
@@ -265,8 +288,8 @@ __global__ void __launch_bounds__((kind_tx(KIND) / 2) * TY) k_batch_flow(
         const int k = q / nitems;
         const int4 item = items[q % nitems];
         const BoxDesc *B = boxes + item.x;
-        const bool ok = run_item<KIND, NF, KIND == KIND_PACKED>(B, item, k % 3, (cur + k) & 1,
-                                                               dts[item.x], zc, scoef, jrun, wrun,
+        const bool ok = run_item<KIND, NF, KIND != KIND_PACKED64>(B, item, k % 3, (cur + k) & 1,
+                                                               steps[item.x].dt, zc, scoef, jrun, wrun,
                                                                smem, dev_error, tmem);
         __syncthreads();  // the column's stores are issued by every thread
         if (threadIdx.x == 0) {
@@ -407,7 +430,7 @@ bool make_plan(int nbox, const int32_t *n, int entropy_mode, Plan &pl, char *why
     pl.off_items = off;
     off = align256(off + sizeof(int4) * pl.nitems);
     pl.off_dt = off;
-    off = align256(off + sizeof(float) * nbox);
+    off = align256(off + sizeof(BoxStep) * nbox);
     pl.off_staging = off;
     off = align256(off + (size_t)nf * maxpts * 8);
     pl.ndiag = diag_blocks(make_layout(1024, 1024, 1024, 4, nf));
@@ -440,7 +463,8 @@ struct gbfd_batch {
     std::vector<BoxDesc> hdesc;
     BoxDesc *ddesc;
     int4 *ditems;
-    float *ddt;
+    BoxStep *dstep;
+    std::vector<Coef<double>> hcoef;  // the boxes' weights in FP64
     char *staging;
     double *dpart, *dout;
     int *derr;
@@ -529,7 +553,7 @@ template <int KIND, int NF>
 cudaError_t launch_substep_k(gbfd_batch *b, int s, int parity, cudaStream_t stream)
 {
     k_batch_substep<KIND, NF><<<grid_of(b), (kind_tx(KIND) / 2) * TY, smem_bytes<KIND, NF>(),
-                                stream>>>(b->ddesc, b->ditems, b->nitems, b->ddt, b->zc, s, parity,
+                                stream>>>(b->ddesc, b->ditems, b->nitems, b->dstep, b->zc, s, parity,
                                           b->derr);
     return cudaGetLastError();
 }
@@ -541,7 +565,7 @@ cudaError_t launch_flow_k(gbfd_batch *b, int nsub, int cur, cudaStream_t stream)
     if (e != cudaSuccess)
         return e;
     k_batch_flow<KIND, NF><<<grid_of(b), (kind_tx(KIND) / 2) * TY, smem_bytes<KIND, NF>(),
-                             stream>>>(b->ddesc, b->ditems, b->nitems, nsub, b->ddt, b->zc, cur,
+                             stream>>>(b->ddesc, b->ditems, b->nitems, nsub, b->dstep, b->zc, cur,
                                        b->dflow, b->derr, b->stall_item);
     return cudaGetLastError();
 }
@@ -610,6 +634,22 @@ gbfd_status graph_for(gbfd_batch *b, int nsteps, cudaGraphExec_t *out, int *nl)
     b->graphs[key] = ex;
     *out = ex;
     return GBFD_OK;
+}
+
+// Every box's time step and folded weights (dt NULL: all zero) to the device.
+cudaError_t upload_steps(gbfd_batch *b, const double *dt)
+{
+    std::vector<BoxStep> h(b->nbox);
+    for (int i = 0; i < b->nbox; ++i) {
+        const double d = dt ? dt[i] : 0.0;
+        h[i].dt = (float)d;
+        h[i].fold = cubic_of(make_fold<float>(b->hcoef[i], d));
+    }
+    cudaError_t e = cudaMemcpyAsync(b->dstep, h.data(), sizeof(BoxStep) * b->nbox,
+                                    cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(b->stream);  // h is a local buffer
+    return e;
 }
 
 gbfd_status check_box(gbfd_batch *b, int box)
@@ -697,7 +737,7 @@ gbfd_status gbfd_batch_init(int nbox, const int32_t *n, const double *lengths, c
     b->cs = cs;
     b->ddesc = (BoxDesc *)(b->ws + pl.off_desc);
     b->ditems = (int4 *)(b->ws + pl.off_items);
-    b->ddt = (float *)(b->ws + pl.off_dt);
+    b->dstep = (BoxStep *)(b->ws + pl.off_dt);
     b->staging = b->ws + pl.off_staging;
     b->dpart = (double *)(b->ws + pl.off_part);
     b->dout = (double *)(b->ws + pl.off_out);
@@ -722,6 +762,8 @@ gbfd_status gbfd_batch_init(int nbox, const int32_t *n, const double *lengths, c
         d.state[1] = (float *)(b->ws + pl.off_state1[i] + d.L.origin);
         d.w = (float *)(b->ws + pl.off_w[i] + d.L.origin);
         d.coef = make_cubic_coef<float>(lengths[i] / n[i], cs, nu[i]);
+        b->hcoef.push_back(make_coef<double>(lengths[i] / n[i], lengths[i] / n[i],
+                                             lengths[i] / n[i], cs, nu[i]));
         bool ok = true;
         for (int wi = 0; wi < 2; ++wi) {
             const int tx = wi ? 64 : 32;
@@ -870,18 +912,12 @@ gbfd_status gbfd_batch_step(gbfd_batch *b, const double *dt, int nsteps)
     }
     if (nsteps == 0)
         return GBFD_OK;
-    std::vector<float> h(b->nbox);
-    for (int i = 0; i < b->nbox; ++i) {
+    for (int i = 0; i < b->nbox; ++i)
         if (!(dt[i] > 0) || !std::isfinite(dt[i])) {
             berr(b, "box %d: dt %g rejected", i, dt[i]);
             return GBFD_ERR_INVALID_ARG;
         }
-        h[i] = (float)dt[i];
-    }
-    cudaError_t e = cudaMemcpyAsync(b->ddt, h.data(), sizeof(float) * b->nbox,
-                                    cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess)
-        e = cudaStreamSynchronize(b->stream);  // h is a local buffer
+    cudaError_t e = upload_steps(b, dt);
     if (e != cudaSuccess)
         return bcuda(b, e, "batch dt upload");
     gbfd_status st;
@@ -1045,11 +1081,7 @@ gbfd_status gbfd_batch_autotune(gbfd_batch *b, int steps, int *best_zc, double *
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return bcuda(b, cudaGetLastError(), "autotune events");
-    std::vector<float> zero(b->nbox, 0.0f);
-    cudaError_t e = cudaMemcpyAsync(b->ddt, zero.data(), sizeof(float) * b->nbox,
-                                    cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess)
-        e = cudaStreamSynchronize(b->stream);
+    cudaError_t e = upload_steps(b, nullptr);
     gbfd_status st = GBFD_OK;
     for (int kind = 0; kind < NKIND && e == cudaSuccess && st == GBFD_OK; ++kind)
         for (int zc : zcs) {

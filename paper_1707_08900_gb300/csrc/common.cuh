@@ -267,6 +267,17 @@ inline FoldCoef<T> make_fold(const Coef<double> &c, double s)
 }
 
 template <class T>
+inline bool fold_is_cubic(const FoldCoef<T> &f)
+{
+    bool iso = f.vc[1] == f.vc[0] && f.vc[2] == f.vc[0];
+    for (int a = 1; a < 3; ++a)
+        for (int k = 0; k < 3; ++k)
+            iso = iso && f.l1[a][k] == f.l1[0][k] && f.n1[a][k] == f.n1[0][k] &&
+                  f.v2[a][k] == f.v2[0][k] && f.x2[a][k] == f.x2[0][k] && f.m3[a][k] == f.m3[0][k];
+    return iso;
+}
+
+template <class T>
 inline FoldCubic<T> cubic_of(const FoldCoef<T> &f)
 {
     FoldCubic<T> q;
@@ -494,6 +505,7 @@ struct StateBufs {
     void *div;   // padded divergence field (19-point form)
     Layout Ls;   // layout of in/out/div (div uses one field)
     Layout Lw;   // layout of w
+    const Coef<double> *cd;  // the box's stencil weights in FP64
     int zc;      // planes per CTA of the default tiled kernel on this grid
 };
 

@@ -516,8 +516,8 @@ cudaError_t launch_lag64_cfg(const StateBufs &b, const Coef<double> &c, const RK
     double *w = (double *)b.w;
     const int skip_plane = st.fault_skip_plane;
     cudaError_t e;
-    const bool iso = coef_is_cubic(c);
     const FoldCoef<double> fc = make_fold<double>(c, st.dt);
+    const bool iso = fold_is_cubic(fc);
     RKStage sd = st;  // the forcing takes the time step too
     for (int a = 0; a < 3; ++a)
         sd.fo.amp[a] *= st.dt;
