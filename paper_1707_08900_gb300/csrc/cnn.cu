@@ -217,18 +217,6 @@ __device__ __forceinline__ void tmem_zero8(uint32_t taddr)
         : "memory");
 }
 
-// Programmatic dependent launch (a kernel launched with programmatic stream
-// serialisation may start while its predecessor in the stream finishes):
-// pdl_wait blocks until the predecessor grid has completed and its memory
-// is visible; pdl_trigger lets this grid's dependant start once every CTA
-// of this grid has triggered or exited.  Both are no-ops for a kernel
-// launched without the attribute.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tiled::smem_u32(bar))
@@ -336,8 +324,8 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     // kernel before this one in the stream, which never writes the weights
     // (the input staging kernel, another convolution or the gradient
     // reduction); the activations it writes are read only below
-    pdl_wait();
-    pdl_trigger();
+    chain_wait();
+    chain_next();
     const int n = a.n;
     const long long n3 = (long long)n * n * n;
     const int nb = (int)(a.npts / n3);
@@ -554,7 +542,7 @@ __global__ void k_input_compact(const float *__restrict__ xs, int nf, int n, int
                                 const float *__restrict__ mean, const float *__restrict__ stdv,
                                 bf16 *__restrict__ x0)
 {
-    pdl_trigger();  // the first convolution may start its prologue
+    chain_next();  // the first convolution may start its prologue
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= npts)
         return;
@@ -572,7 +560,7 @@ __global__ void k_input_state(const float *__restrict__ st, Layout L, int nf, in
                               const float *__restrict__ mean, const float *__restrict__ stdv,
                               bf16 *__restrict__ x0)
 {
-    pdl_trigger();  // the first convolution may start its prologue
+    chain_next();  // the first convolution may start its prologue
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = L.nx;
     if (p >= n * n * n)
@@ -589,7 +577,7 @@ __global__ void k_input_state(const float *__restrict__ st, Layout L, int nf, in
 __global__ void k_apply(float *__restrict__ st, Layout L, int nf, const float *__restrict__ y,
                         const float *__restrict__ sout)
 {
-    pdl_wait();  // launched to overlap the last convolution's tail
+    chain_wait();  // launched to overlap the last convolution's tail
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = L.nx;
     if (p >= n * n * n)

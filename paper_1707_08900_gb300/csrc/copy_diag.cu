@@ -164,6 +164,8 @@ template <class T>
 __global__ void __launch_bounds__(256) k_fill_ghosts_z(T *__restrict__ origin, Layout L, int nf,
                                                       int odd_mask)
 {
+    chain_wait();
+    chain_next();
     constexpr int V = 16 / sizeof(T);
     const long long pv = L.plane / V;  // 16-byte vectors per plane
     const long long total = (long long)nf * 2 * GZW * pv;
@@ -201,12 +203,12 @@ cudaError_t launch_fill_ghosts_z(void *origin, const Layout &L, int nf, int odd_
         return cudaSuccess;
     const long long total = (long long)nf * 2 * GZW * (L.plane * L.w / 16);
     const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-    if (L.w == 8)
-        k_fill_ghosts_z<double><<<blocks, 256, 0, stream>>>((double *)origin, L, nf, odd_mask);
-    else
-        k_fill_ghosts_z<float><<<blocks, 256, 0, stream>>>((float *)origin, L, nf, odd_mask);
     *launches += 1;
-    return cudaGetLastError();
+    if (L.w == 8)
+        return launch_chained<k_fill_ghosts_z<double>>(dim3(blocks), dim3(256), 0, false, stream,
+                                                       (double *)origin, L, nf, odd_mask);
+    return launch_chained<k_fill_ghosts_z<float>>(dim3(blocks), dim3(256), 0, false, stream,
+                                                  (float *)origin, L, nf, odd_mask);
 }
 
 namespace {
@@ -339,9 +341,9 @@ namespace {
 __global__ void k_forcing_tables(int kx, int ky, int kz, double cphi, double sphi, int nx, int ny,
                                  int nz, double2 *__restrict__ tab, float2 *__restrict__ tab32)
 {
+    // the kernels of the step before still read the tables: only the phases
+    // are formed ahead of them
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nx + ny + nz)
-        return;
     int n, k, idx;
     if (i < nx) {
         n = nx, k = kx, idx = i;
@@ -360,6 +362,10 @@ __global__ void k_forcing_tables(int kx, int ky, int kz, double cphi, double sph
         cs = c2;
         sn = s2;
     }
+    chain_wait();
+    chain_next();
+    if (i >= nx + ny + nz)
+        return;
     tab[i] = make_double2(cs, sn);
     tab32[i] = make_float2((float)cs, (float)sn);
 }
@@ -371,10 +377,9 @@ cudaError_t launch_forcing_tables(int kx, int ky, int kz, double phi, int nx, in
                                   int *launches)
 {
     const int n = nx + ny + nz;
-    k_forcing_tables<<<(n + 255) / 256, 256, 0, stream>>>(kx, ky, kz, cos(phi), sin(phi), nx, ny,
-                                                           nz, tab, tab32);
     *launches += 1;
-    return cudaGetLastError();
+    return launch_chained<k_forcing_tables>(dim3((n + 63) / 64), dim3(64), 0, false, stream, kx, ky,
+                                            kz, cos(phi), sin(phi), nx, ny, nz, tab, tab32);
 }
 
 int diag_blocks(const Layout &L)

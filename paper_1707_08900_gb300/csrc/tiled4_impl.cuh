@@ -152,8 +152,8 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
     if constexpr (FORCE) {
         // the column's x-y phase factor of the forcing, Re/Im of tx[x] ty[y]
         if (valid0) {
-            const float2 a0 = __ldg(fo->tx32 + x), a1 = __ldg(fo->tx32 + x + 1);
-            const float2 b = __ldg(fo->ty32 + y);
+            const float2 a0 = fo->tx32[x], a1 = fo->tx32[x + 1];
+            const float2 b = fo->ty32[y];
             fxy0 = make_float2(a0.x * b.x - a0.y * b.y, a0.x * b.y + a0.y * b.x);
             fxy1 = make_float2(a1.x * b.x - a1.y * b.y, a1.x * b.y + a1.y * b.x);
         }
@@ -505,7 +505,7 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
             r[3] = P::add(r[3], acz[S]);
             if constexpr (FORCE) {
                 // f_i = amp_i cos(k.x + phi) (amp folded like the weights)
-                const float2 cz = __ldg(fo->tz32 + z0 + o);
+                const float2 cz = fo->tz32[z0 + o];
                 const V fc = P::mk(fxy0.x * cz.x - fxy0.y * cz.y, fxy1.x * cz.x - fxy1.y * cz.y);
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
@@ -722,6 +722,8 @@ __global__ void __launch_bounds__((TX / 2) * TY, MINB) k_substep_lag(
         tc::fence_after_sync();
         tmem = *reinterpret_cast<volatile uint32_t *>(slot);
     }
+    chain_wait();
+    chain_next();
     const int x0 = (blockIdx.x % tiles_x) * TX;
     const int y0 = (blockIdx.x / tiles_x) * TY;
     const int z0 = blockIdx.y * zc;
@@ -761,7 +763,7 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
     const dim3 block((TX / 2) * TY);
     float *out = (float *)b.out;
     TW *w = (TW *)b.w;
-    cudaError_t e;
+    cudaError_t e = cudaErrorNotSupported;
     // the weights with the time step folded in where the update is FP32 (the
     // precision forms multiply by dt in their own arithmetic); equal spacing
     // on every axis: the isotropic set (same values)
@@ -776,14 +778,11 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
             sd.fo.amp32[a] = (float)(st.fo.amp[a] * st.dt);
 #define GBFD_LAUNCH_LAG_C(NFV, FRC, CT, CV)                                                       \
     do {                                                                                          \
-        auto kern = tiled4::k_substep_lag<TW, TA, NFV, TX, TY, NS, U, MINB, ICVT, FRC, TM, CT,    \
-                                          SHFL>;                                                  \
+        constexpr auto kern = tiled4::k_substep_lag<TW, TA, NFV, TX, TY, NS, U, MINB, ICVT, FRC,  \
+                                                    TM, CT, SHFL>;                                \
         constexpr int sm = tiled4::RingL<TW, NFV, TX, TY, NS, U>::BYTES;                          \
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);          \
-        if (e != cudaSuccess)                                                                     \
-            return e;                                                                             \
-        kern<<<grid, block, sm, stream>>>(*map, *wmap, out, w, b.Ls, b.Lw, CV, sd, zc, tiles_x,   \
-                                          dev_error, skip_plane);                                 \
+        e = launch_chained<kern>(grid, block, sm, false, stream, *map, *wmap, out, w, b.Ls, b.Lw, \
+                                 CV, sd, zc, tiles_x, dev_error, skip_plane);                     \
     } while (0)
 #define GBFD_LAUNCH_LAG(NFV, FRC)                                                                 \
     do {                                                                                          \
@@ -808,14 +807,11 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
         if (nf == 5 && frc_ok && iso && full && st.s >= 0 && st.s <= 2) {
 #define GBFD_LAUNCH_LAG_S(FRC, SV)                                                                \
     do {                                                                                          \
-        auto kern = tiled4::k_substep_lag<TW, TA, 5, TX, TY, NS, U, MINB, ICVT, FRC, TM,          \
-                                          FoldCubic<float>, SHFL, SV, true>;                      \
+        constexpr auto kern = tiled4::k_substep_lag<TW, TA, 5, TX, TY, NS, U, MINB, ICVT, FRC,    \
+                                                    TM, FoldCubic<float>, SHFL, SV, true>;        \
         constexpr int sm = tiled4::RingL<TW, 5, TX, TY, NS, U>::BYTES;                            \
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);          \
-        if (e != cudaSuccess)                                                                     \
-            return e;                                                                             \
-        kern<<<grid, block, sm, stream>>>(*map, *wmap, out, w, b.Ls, b.Lw, cc, sd, zc, tiles_x,   \
-                                          dev_error, skip_plane);                                 \
+        e = launch_chained<kern>(grid, block, sm, false, stream, *map, *wmap, out, w, b.Ls, b.Lw, \
+                                 cc, sd, zc, tiles_x, dev_error, skip_plane);                     \
     } while (0)
 #define GBFD_LAUNCH_LAG_SS(FRC)                                                                   \
     do {                                                                                          \
@@ -835,7 +831,7 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
 #undef GBFD_LAUNCH_LAG_SS
 #undef GBFD_LAUNCH_LAG_S
             *launches += 1;
-            return cudaGetLastError();
+            return e;
         }
     }
     if (nf == 5) {
@@ -852,7 +848,7 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
 #undef GBFD_LAUNCH_LAG
 #undef GBFD_LAUNCH_LAG_C
     *launches += 1;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace gbfd

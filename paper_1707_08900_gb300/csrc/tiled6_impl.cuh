@@ -126,6 +126,8 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
     tc::fence_after_sync();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(tslot);
     const uint32_t trow = tmem + ((uint32_t)(threadIdx.x & ~31) << 16);
+    chain_wait();
+    chain_next();
 
     const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
     const int x0 = (blockIdx.x % tiles_x) * TX;
@@ -523,16 +525,10 @@ cudaError_t launch_lag64_cfg(const StateBufs &b, const Coef<double> &c, const RK
         sd.fo.amp[a] *= st.dt;
 #define GBFD_LAUNCH_L64_F(NFV, FRC, CT, CV)                                                       \
     do {                                                                                          \
-        auto kern = tiled6::k_substep_lag64<NFV, TX, TY, NS, MINB, FRC, CT>;                      \
+        constexpr auto kern = tiled6::k_substep_lag64<NFV, TX, TY, NS, MINB, FRC, CT>;            \
         constexpr int sm = tiled6::Ring64<NFV, TX, TY, NS>::BYTES;                                \
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);          \
-        if (e == cudaSuccess)                                                                     \
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,        \
-                                     (int)cudaSharedmemCarveoutMaxShared);                        \
-        if (e != cudaSuccess)                                                                     \
-            return e;                                                                             \
-        kern<<<grid, block, sm, stream>>>(*map, out, w, b.Ls, b.Lw, CV, sd, zc, tiles_x,          \
-                                          dev_error, skip_plane);                                 \
+        e = launch_chained<kern>(grid, block, sm, true, stream, *map, out, w, b.Ls, b.Lw, CV, sd, \
+                                 zc, tiles_x, dev_error, skip_plane);                             \
     } while (0)
 #define GBFD_LAUNCH_L64(NFV, CT, CV)                                                              \
     do {                                                                                          \
@@ -555,7 +551,7 @@ cudaError_t launch_lag64_cfg(const StateBufs &b, const Coef<double> &c, const RK
 #undef GBFD_LAUNCH_L64
 #undef GBFD_LAUNCH_L64_F
     *launches += 1;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace gbfd
