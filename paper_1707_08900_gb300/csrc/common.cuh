@@ -418,6 +418,15 @@ __device__ __forceinline__ void rk3_update<ffloat, float, float>(bool first, ffl
     rk3_update_ff(first, alpha, beta, dt, r.hi, u, w, out);
 }
 
+// The FP64 update of Eq. 10 (FP32 storage) reached through float-float
+// arithmetic: carries the coefficient in both forms.
+struct fexact {
+    ffloat f;
+    double d;
+    __host__ __device__ fexact() : d(0.0) {}
+    __host__ __device__ fexact(double v) : f(v), d(v) {}
+};
+
 // Exact IEEE-754 conversions between binary32 and binary64 done with integer
 // instructions, so that GB300's narrow FP64 pipe is left to the arithmetic.
 // binary32 (sign, 8-bit exponent e, 23-bit fraction m) -> binary64: exponent
@@ -470,6 +479,80 @@ __device__ __forceinline__ void rk3_update_f64(bool first, double alpha, double 
     else
         w = down(wn);
     out = down(fma(beta, wn, up(u)));
+}
+
+// rk3_update_ff for two points at once in packed FP32x2 instructions (the same
+// operations and bits; constants are broadcast pairs, n* negated ones, so that
+// error terms come out negated by one fused multiply-add).
+//
+// CHECK: `safe` tells, per point, whether both results are also those of the
+// FP64 update (rk3_update_f64).  The float-float value and the FP64 one differ
+// by less than E = 2^-43 M + 2^-146, M the sum of the magnitudes of the terms
+// added (float-float: 2^-46 M by Dekker's and Knuth's bounds, FP64: 2^-52 M; the
+// constant covers products whose error terms leave the binary32 range), so
+// when the lowest and the highest value within E round to the same binary32
+// number, so does the FP64 one.  M = 0 is exact.  Infinities and NaN fail the
+// comparison.  About 4 in 10^6 values do; they take the FP64 update.
+struct FfConst {
+    float2 dh, ndh, ndl, ah, nah, nal, bh, nbh, nbl;
+    __device__ __forceinline__ FfConst(const ffloat &dt, const ffloat &a, const ffloat &b)
+        : dh(make_float2(dt.hi, dt.hi)), ndh(make_float2(-dt.hi, -dt.hi)),
+          ndl(make_float2(-dt.lo, -dt.lo)), ah(make_float2(a.hi, a.hi)),
+          nah(make_float2(-a.hi, -a.hi)), nal(make_float2(-a.lo, -a.lo)),
+          bh(make_float2(b.hi, b.hi)), nbh(make_float2(-b.hi, -b.hi)),
+          nbl(make_float2(-b.lo, -b.lo))
+    {
+    }
+};
+template <bool CHECK>
+__device__ __forceinline__ void rk3_pair_ff(const bool first, const FfConst &c, const float2 r,
+                                            const float2 u, float2 &w, float2 &out, bool &safe0,
+                                            bool &safe1)
+{
+    const float2 N1 = make_float2(-1.f, -1.f);
+    auto sub = [&](float2 a, float2 b) { return __ffma2_rn(b, N1, a); };
+    auto two_sum2 = [&](float2 a, float2 b, float2 &s, float2 &e) {
+        s = __fadd2_rn(a, b);
+        const float2 bb = sub(s, a);
+        e = __fadd2_rn(sub(a, sub(s, bb)), sub(b, bb));
+    };
+    // negated errors of the products: -(a b - p) = (-a) b + p
+    const float2 p2 = __fmul2_rn(c.dh, r);
+    const float2 n2 = __ffma2_rn(c.ndl, r, __ffma2_rn(c.ndh, r, p2));
+    float2 hi, lo, m;
+    if (CHECK)
+        m = make_float2(fabsf(p2.x), fabsf(p2.y));
+    if (first) {
+        hi = sub(p2, n2);
+        lo = __fmul2_rn(__fadd2_rn(n2, sub(hi, p2)), N1);
+    } else {
+        const float2 p1 = __fmul2_rn(c.ah, w);
+        const float2 n1 = __ffma2_rn(c.nal, w, __ffma2_rn(c.nah, w, p1));
+        float2 s, t;
+        two_sum2(p1, p2, s, t);
+        two_sum2(s, sub(t, __fadd2_rn(n1, n2)), hi, lo);
+        if (CHECK)
+            m = make_float2(m.x + fabsf(p1.x), m.y + fabsf(p1.y));
+    }
+    const float2 q = __fmul2_rn(c.bh, hi);
+    float2 nf = __ffma2_rn(c.nbh, hi, q);
+    nf = __ffma2_rn(c.nbh, lo, nf);
+    nf = __ffma2_rn(c.nbl, hi, nf);
+    float2 s2, t2;
+    two_sum2(u, q, s2, t2);
+    const float2 g = sub(t2, nf);
+    out = __fadd2_rn(s2, g);
+    w = hi;
+    if (CHECK) {
+        const float2 C = make_float2(0x1p-43f, 0x1p-43f), K = make_float2(0x1p-146f, 0x1p-146f);
+        const float2 e = __ffma2_rn(C, m, K);
+        const float2 wa = __fadd2_rn(hi, __fadd2_rn(lo, e)), wb = __fadd2_rn(hi, sub(lo, e));
+        const float2 mo = make_float2(fabsf(q.x) + fabsf(u.x), fabsf(q.y) + fabsf(u.y));
+        const float2 eo = __ffma2_rn(C, mo, __ffma2_rn(c.bh, e, K));
+        const float2 oa = __fadd2_rn(s2, __fadd2_rn(g, eo)), ob = __fadd2_rn(s2, sub(g, eo));
+        safe0 = (wa.x == wb.x || m.x == 0.f) && (oa.x == ob.x || mo.x == 0.f);
+        safe1 = (wa.y == wb.y || m.y == 0.f) && (oa.y == ob.y || mo.y == 0.f);
+    }
 }
 
 // Store v at interior (x, y, z) of field f and at its periodic ghost copies.

@@ -84,6 +84,12 @@ cudaError_t launch_lag_shfl(const StateBufs &b, const Coef<float> &c, const RKSt
                             int zc, int cfg_key, int *dev_error, TmapCache *cache,
                             cudaStream_t stream, int *launches);
 
+// The FP64-update precision form (u-tilde in FP32, 55-point form) on the FP32
+// default kernel (tiled_ff.cu).
+cudaError_t launch_lag_exact(const StateBufs &b, const Coef<float> &c, const RKStage &st, int nf,
+                             int zc, int *dev_error, TmapCache *cache, cudaStream_t stream,
+                             int *launches);
+
 template <class TS, class TW, class TA>
 cudaError_t launch_substep_tiled(const StateBufs &b, const Coef<TS> &c, const RKStage &st, int nf,
                                  int form, int cfg, int *dev_error, TmapCache *cache,

@@ -211,6 +211,17 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
     for (int m = 0; m < W; ++m)
         acx[m] = acy[m] = acz[m] = P::bc(0.f);
 
+    // the float-float constants of the precision forms
+    const FfConst ffc = [&] {
+        if constexpr (std::is_same<TA, fexact>::value)
+            return FfConst(dt.f, alpha.f, beta.f);
+        else if constexpr (std::is_same<TA, ffloat>::value)
+            return FfConst(dt, alpha, beta);
+        else
+            return FfConst(ffloat(), ffloat(), ffloat());
+    }();
+    (void)ffc;
+
     const V NEG1 = P::bc(-1.f);
     // add the arm differences d[k-1] of one plane, ac index MC, with weights
     // M3(pair, k): plus to the outputs below it, minus to those above
@@ -522,16 +533,31 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
                     o2 = P::fma(BETA, wn, u0);
                     if (!last)
                         *reinterpret_cast<V *>(w + f * Lw.fpitch + go_w) = wn;
-                } else if constexpr (std::is_same<TA, ffloat>::value) {
-                    // the precision form in float-float arithmetic
+                } else if constexpr (std::is_same<TA, ffloat>::value ||
+                                     std::is_same<TA, fexact>::value) {
+                    // the precision forms' update in float-float arithmetic;
+                    // fexact: where that might round differently, in FP64
                     static_assert(std::is_same<TW, float>::value, "u-tilde stored in FP32");
-                    float wo[2] = {first ? 0.f : wv[f].x, first ? 0.f : wv[f].y};
-                    float on[2];
-                    rk3_update_ff(first, alpha, beta, dt, r[f].x, u0.x, wo[0], on[0]);
-                    rk3_update_ff(first, alpha, beta, dt, r[f].y, u0.y, wo[1], on[1]);
-                    o2 = make_float2(on[0], on[1]);
+                    V wn = first ? P::bc(0.f) : wv[f];
+                    const V wold = wn;
+                    bool safe0 = true, safe1 = true;
+                    if constexpr (std::is_same<TA, fexact>::value) {
+                        rk3_pair_ff<true>(first, ffc, r[f], u0, wn, o2, safe0, safe1);
+                        if (!safe0) {
+                            wn.x = wold.x;
+                            rk3_update_f64<true, float>(first, alpha.d, beta.d, dt.d, r[f].x, u0.x,
+                                                        wn.x, o2.x);
+                        }
+                        if (!safe1) {
+                            wn.y = wold.y;
+                            rk3_update_f64<true, float>(first, alpha.d, beta.d, dt.d, r[f].y, u0.y,
+                                                        wn.y, o2.y);
+                        }
+                    } else {
+                        rk3_pair_ff<false>(first, ffc, r[f], u0, wn, o2, safe0, safe1);
+                    }
                     if (!last)
-                        *reinterpret_cast<V *>(w + f * Lw.fpitch + go_w) = make_float2(wo[0], wo[1]);
+                        *reinterpret_cast<V *>(w + f * Lw.fpitch + go_w) = wn;
                 } else {
                     static_assert(std::is_same<TA, double>::value, "FP64 update");
                     TW wo[2] = {first ? (TW)0 : wv[f].x, first ? (TW)0 : wv[f].y};
@@ -798,7 +824,8 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
     // arithmetic included): the substep is a template argument and the
     // grid-extent test goes
     constexpr bool SPEC = TM && MINB == 1 && !ICVT && !SHFL && std::is_same<TW, float>::value &&
-                          (std::is_same<TA, float>::value || std::is_same<TA, ffloat>::value);
+                          (std::is_same<TA, float>::value || std::is_same<TA, ffloat>::value ||
+                           std::is_same<TA, fexact>::value);
     const bool full = b.Ls.nx % TX == 0 && b.Ls.ny % TY == 0;
     if constexpr (SPEC) {
         // forced steps too, in FP32 arithmetic (the forcing is a compile-time

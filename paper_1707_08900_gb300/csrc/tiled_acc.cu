@@ -14,8 +14,16 @@ cudaError_t launch_substep_tiled(const StateBufs &b, const Coef<TS> &c, const RK
                                  int form, int cfg, int *dev_error, TmapCache *cache,
                                  cudaStream_t stream, int *launches)
 {
-    // default: the packed kernel with integer conversions, z-chunk 32 (its
-    // FP64 update binds; 40-plane chunks measured 3% slower here)
+    // default of the 55-point form with u-tilde in FP32: the FP32 default kernel,
+    // its update in float-float arithmetic with the few results that could
+    // round differently redone in FP64 (the same bits as the FP64 update of the
+    // same right-hand side, without its 15 FP64 operations per point on a pipe
+    // of 2 lanes per SM and clock): 1179 -> 475 us per substep at 256^3
+    if constexpr (sizeof(TW) == 4)
+        if (cfg < 0 && form == 0)
+            return launch_lag_exact(b, c, st, nf, b.zc, dev_error, cache, stream, launches);
+    // else the packed kernel with integer conversions, z-chunk 32 (its FP64
+    // update binds; 40-plane chunks measured 3% slower here)
     const int idx = cfg < 0 ? 1 : cfg;
     const TileConfig t = tiled_config(4, idx % kZcChoices);
     cudaError_t e;
