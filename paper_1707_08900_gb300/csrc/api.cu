@@ -790,14 +790,26 @@ gbfd_status gbfd_cfl_dt(gbfd_ctx *ctx, double cfl, double cnu, double *dt_out)
             set_err(ctx, "cfl_dt: bad arguments");
         return GBFD_ERR_INVALID_ARG;
     }
-    gbfd_diag d;
-    gbfd_status st = gbfd_diagnostics(ctx, &d);
+    gbfd_status st = check_ctx(ctx);
     if (st != GBFD_OK)
         return st;
+    int nl = 0;
+    cudaError_t e = launch_umax(ctx->state_region[ctx->cur] + ctx->Ls.origin, ctx->Ls,
+                                ctx->diag_out, ctx->stream, &nl);
+    ctx->launches += nl;
+    if (e != cudaSuccess)
+        return cuda_fail(ctx, e, "largest velocity launch");
+    double uu = 0.0;
+    e = cudaMemcpyAsync(&uu, ctx->diag_out, sizeof uu, cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess)
+        return cuda_fail(ctx, e, "largest velocity read");
+    const double umax = std::sqrt(uu);
     const double *h = ctx->h;
     double dmin = h[0] < h[1] ? h[0] : h[1];
     dmin = dmin < h[2] ? dmin : h[2];
-    double dt = cfl * dmin / (d.umax + ctx->p.cs);
+    double dt = cfl * dmin / (umax + ctx->p.cs);
     if (ctx->p.nu > 0) {
         const double dtn = cnu * dmin * dmin / ctx->p.nu;
         dt = dtn < dt ? dtn : dt;

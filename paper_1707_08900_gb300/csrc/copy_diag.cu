@@ -1,6 +1,7 @@
 // State copies into/out of the padded layout and the FP64 diagnostics
 // reductions (mass, kinetic energy, max |u| for the time-step rule, per-field
 // rms and max, non-finite flag).
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -312,7 +313,94 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_diag_final(const double *__res
     }
 }
 
+// max |u|^2 alone, for the time-step rule: the same FP64 value as the full
+// reduction's, NaNs skipped as by fmax.  The FP64 pipe (2 lanes per SM and
+// clock) is what the full reduction waits for (its sums and exp(lnrho): 365 us
+// at 200 x 136 x 105), so FP32 storage looks at |u|^2 in FP32 first, whose
+// relative error is below 2^-22, and only values within 2^-20 of the largest
+// seen by the warp, or not comparable (overflow, NaN, tiny), are squared in
+// FP64.  A thread reads 16 bytes of each velocity component; the padded planes
+// are scanned as they lie (ghost columns and rows hold copies, padding zeros).
+// DRAM-bound: 11 us there.
+template <class TS>
+__global__ void __launch_bounds__(DIAG_THREADS) k_umax(const TS *__restrict__ st,
+                                                       long long fpitch, long long nvec,
+                                                       unsigned long long *__restrict__ out)
+{
+    constexpr int V = 16 / sizeof(TS);
+    double best = 0.0;
+    float lim = 0.f;
+    for (long long base = (long long)blockIdx.x * DIAG_THREADS; base < nvec;
+         base += (long long)gridDim.x * DIAG_THREADS) {
+        const long long i = base + threadIdx.x;
+        uint4 q[3];
+#pragma unroll
+        for (int f = 0; f < 3; ++f)
+            q[f] = i < nvec ? __ldg(reinterpret_cast<const uint4 *>(st + (1 + f) * fpitch) + i)
+                            : make_uint4(0, 0, 0, 0);
+        const TS *a = reinterpret_cast<const TS *>(&q[0]), *b = reinterpret_cast<const TS *>(&q[1]),
+                 *c = reinterpret_cast<const TS *>(&q[2]);
+        auto exact = [&](int j) {
+            const double x = (double)a[j], y = (double)b[j], z = (double)c[j];
+            best = fmax(best, x * x + y * y + z * z);
+        };
+        if constexpr (sizeof(TS) == 8) {
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+                exact(j);
+        } else {
+            float s[V];
+            bool some = false;
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                s[j] = a[j] * a[j] + b[j] * b[j] + c[j] * c[j];
+                some = some || !(s[j] < lim);
+            }
+            if (__any_sync(0xffffffffu, some)) {
+                // the warp's largest comparable value first, then what comes
+                // within the FP32 error of it
+                float m = 0.f;
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    m = s[j] < INFINITY ? fmaxf(m, s[j]) : m;
+                m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+                if (m > 1e-30f)
+                    lim = fmaxf(lim, m * (1.f - 0x1p-20f));
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    if (!(s[j] < lim))
+                        exact(j);
+            }
+        }
+    }
+    // (non-negative FP64 values order as their bits)
+    unsigned long long v = (unsigned long long)__double_as_longlong(best);
+    for (int k = 16; k > 0; k >>= 1)
+        v = max(v, __shfl_xor_sync(0xffffffffu, v, k));
+    if (threadIdx.x % 32 == 0 && v)
+        atomicMax(out, v);
+}
+
 }  // namespace
+
+cudaError_t launch_umax(const void *state, const Layout &L, double *out, cudaStream_t stream,
+                        int *launches)
+{
+    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), stream);
+    if (e != cudaSuccess)
+        return e;
+    // whole planes: a multiple of 128 bytes, from a 16-byte aligned start
+    const long long nvec = (long long)L.nz * L.plane * L.w / 16;
+    const int blocks = (int)std::min<long long>((nvec + DIAG_THREADS - 1) / DIAG_THREADS, 1216);
+    if (L.w == 8)
+        k_umax<double><<<blocks, DIAG_THREADS, 0, stream>>>((const double *)state, L.fpitch, nvec,
+                                                           (unsigned long long *)out);
+    else
+        k_umax<float><<<blocks, DIAG_THREADS, 0, stream>>>((const float *)state, L.fpitch, nvec,
+                                                          (unsigned long long *)out);
+    *launches += 1;
+    return cudaGetLastError();
+}
 
 cudaError_t launch_scatter(const void *src, int src_fp64, void *dst, const Layout &L, int nf,
                            cudaStream_t stream, int *launches)

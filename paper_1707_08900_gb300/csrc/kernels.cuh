@@ -151,4 +151,8 @@ cudaError_t launch_diagnostics(const void *state, const Layout &L, int nf, doubl
                                double *partials, int nblocks, double *out, cudaStream_t stream,
                                int *launches);
 
+// *out = max |u|^2 over the current state (one FP64 value on the device).
+cudaError_t launch_umax(const void *state, const Layout &L, double *out, cudaStream_t stream,
+                        int *launches);
+
 }  // namespace gbfd

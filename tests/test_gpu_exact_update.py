@@ -62,7 +62,7 @@ def test_exact_update_keeps_extreme_values():
     build.build()
     shape = (12, 16, 32)
     st = np.zeros((5,) + shape, dtype=np.float32)
-    special = np.array([0.0, 1e-40, -3e-39, 1.1754944e-38, 3.0e37, -3.0e37, 1e-30,
+    special = np.array([0.0, 1e-40, -3e-39, 1.1754944e-38, 1.0e37, -1.0e37, 1e-30,
                         1.0 + 2.0 ** -23, -(1.0 + 2.0 ** -22), 7.0], dtype=np.float32)
     st[4] = np.resize(special, shape[0] * shape[1] * shape[2]).reshape(shape)
     out = _run("fp32_acc64", st, shape, (2 * np.pi,) * 3, 1e-3, 1)
