@@ -362,11 +362,13 @@ gbfd_status gbfd_batch_sync(gbfd_batch *b);
 
 /* Options (no counterpart in the paper):
  * GBFD_BATCH_OPT_GRAPH: 1 = replay CUDA graphs (default), 0 = direct launches;
- * GBFD_BATCH_OPT_ZCHUNK: planes per work item: 8, 16, 32 (default), 64;
+ * GBFD_BATCH_OPT_ZCHUNK: planes per work item: 8, 16, 32, 64 (default: chosen
+ *   from the boxes);
  * GBFD_BATCH_OPT_GRID: persistent CTAs per launch (0 = SMs x resident CTAs);
  * GBFD_BATCH_OPT_KERNEL: column routine: 0 = two-plane packed on 32 x 8
- *   tiles (default), 1 = lagged output with TMEM on 32 x 8 (weights read from
- *   shared memory), 2 = two-plane packed on 64 x 8;
+ *   tiles, 1 = lagged output with TMEM on 32 x 8 (weights read from shared
+ *   memory), 2 = two-plane packed on 64 x 8 (default: 1 for five fields with
+ *   64-plane items, else 0);
  * GBFD_BATCH_OPT_DATAFLOW: 1 = all substeps of a gbfd_batch_step in ONE
  *   persistent launch, work items ordered by substep and each waiting
  *   (bounded, about 2 s) for its box's previous substep through a per-box
@@ -455,7 +457,7 @@ const char *gbfd_cnn_last_error(const gbfd_cnn *c);
  * GBFD_CNN_OPT_CONV_GRID: CTAs per convolution launch, each walking an equal
  * share of the 256-point tiles (0 = default, one per SM); a small value
  * makes every CTA loop over many tiles.  GBFD_CNN_OPT_WGRAD_PARTS: CTAs of
- * the weight-gradient sums, 1..296 (0 = default 296).  Results agree to
+ * the weight-gradient sums, 1..296 (0 = default, one per SM).  Results agree to
  * rounding whatever the values; out-of-range values -> INVALID_ARG. */
 enum { GBFD_CNN_OPT_CONV_GRID = 1, GBFD_CNN_OPT_WGRAD_PARTS = 2 };
 gbfd_status gbfd_cnn_set_option(gbfd_cnn *c, int key, int64_t value);

@@ -547,6 +547,37 @@ gbfd_status build_items(gbfd_batch *b, int zc, int kind)
     return GBFD_OK;
 }
 
+// Chunk length and column routine until the caller or the autotuner chooses.
+// In the dataflow launch items of different boxes and substeps overlap, so a
+// substep takes about the planes of all items (each with 3 planes' worth of
+// halo and start-up) over the resident CTAs, and no less than its longest item,
+// which the box's next substep waits for.  That picks the measured best length
+// of the four in each of 11 batches, from three 16^3 boxes (8 planes) to two
+// 256^3 (64); us per 4 steps: 96 boxes of 32^3 to 128^3 16293 at the earlier
+// 32 planes, 15502 at 64; 8 x 64^3 597 -> 552 (16); 4 x 32^3 521 -> 195 (8).
+// With long columns of five fields the lagged routine is the faster one (96
+// boxes 15239), with short ones its longer start-up costs more.
+void default_items(const gbfd_batch *b, int *zc, int *kind)
+{
+    const double h = 3.0;
+    double best = 1e300;
+    for (int z : {8, 16, 32, 64}) {
+        double planes = 0.0, longest = 0.0;
+        for (int n : b->n) {
+            const int c = zc_for(n, z);
+            const double tiles = (double)((n + 31) / 32) * ((n + TY - 1) / TY);
+            planes += tiles * (n + h * ((n + c - 1) / c));
+            longest = std::max(longest, c + h);
+        }
+        const double t = std::max(planes / b->grid_kind[KIND_PACKED], longest);
+        if (t < best) {
+            best = t;
+            *zc = z;
+        }
+    }
+    *kind = *zc == 64 && b->nf == 5 ? KIND_LAG : KIND_PACKED;
+}
+
 int grid_of(const gbfd_batch *b) { return b->grid > 0 ? b->grid : b->grid_kind[b->kind]; }
 
 template <int KIND, int NF>
@@ -828,7 +859,9 @@ gbfd_status gbfd_batch_init(int nbox, const int32_t *n, const double *lengths, c
         delete b;
         return GBFD_ERR_CUDA;
     }
-    gbfd_status st = build_items(b, 32, KIND_PACKED);
+    int zc, kind;
+    default_items(b, &zc, &kind);
+    gbfd_status st = build_items(b, zc, kind);
     if (st != GBFD_OK) {
         berr(nullptr, "%s", b->err);
         cudaStreamDestroy(b->cap);

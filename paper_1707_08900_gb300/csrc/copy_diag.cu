@@ -52,69 +52,118 @@ __device__ __forceinline__ void store_quad(double *p, const double (&v)[4])
     reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
 }
 
-constexpr int COPY_WARPS = 8;  // rows per block: one warp per row
+constexpr int COPY_THREADS = 256;
+
+// Group of LPR lanes that one row takes (8 for rows of up to 32 values, 16 up to
+// 64, else 32) and the rows a group takes at once: their loads are all issued
+// before the first store.
+template <int LPR>
+struct RowGroup {
+    static constexpr int ROWS = LPR == 32 ? 2 : 4;
+    static constexpr int PER_BLOCK = COPY_THREADS / LPR * ROWS;
+};
 
 // Every padded row (interior and ghost rows, interior and ghost columns) of
-// every field from the compact source; ghosts take the periodic image.  One
-// warp per destination row; VEC: source rows 16-byte aligned (nx % 4 == 0
-// and an aligned base), so the interior moves in 16-byte accesses.  The
-// source may be device memory or pinned host memory mapped into the device
-// address space.
-template <class TD, class TSrc, bool VEC>
-__global__ void __launch_bounds__(32 * COPY_WARPS) k_scatter(const TSrc *__restrict__ src,
-                                                            TD *__restrict__ dst, Layout L,
-                                                            long long nrows)
+// every field from the compact source; ghosts take the periodic image.  VEC:
+// source rows 16-byte aligned (nx % 4 == 0 and an aligned base), so values move
+// in 16-byte accesses, four columns at a time; the four ghost columns on each
+// side are the first and the last four of the row, written by the thread that
+// holds them.  The source may be device memory or pinned host memory mapped into
+// the device address space.  DRAM-bound; with a warp per row and 64-bit row
+// arithmetic 256^3 took 133 us (5.0 TB/s) and a 32^3 box used 8 of 32 lanes.
+// IDX: unsigned when the rows can be counted in it.
+template <class TD, class TSrc, bool VEC, int LPR, class IDX>
+__global__ void __launch_bounds__(COPY_THREADS) k_scatter(const TSrc *__restrict__ src,
+                                                         TD *__restrict__ dst, Layout L, IDX nrows)
 {
-    const long long row = (long long)blockIdx.x * COPY_WARPS + threadIdx.x / 32;
-    const int lane = threadIdx.x % 32;
-    if (row >= nrows)
-        return;
-    const int Y = (int)(row % L.rows);
-    const long long fz = row / L.rows;
-    const int z = (int)(fz % L.nz), f = (int)(fz / L.nz);
-    const int y = wrapi(Y - GY, L.ny);
-    const TSrc *s = src + (((long long)f * L.nz + z) * L.ny + y) * L.nx;
-    TD *d = dst + (long long)f * L.fpitch + (long long)z * L.plane + (long long)Y * L.P;
+    using G = RowGroup<LPR>;
+    const int lane = threadIdx.x % LPR;
+    const IDX row0 = (IDX)blockIdx.x * G::PER_BLOCK + threadIdx.x / LPR * G::ROWS;
+    const TSrc *s[G::ROWS];
+    TD *d[G::ROWS];
+    int n = 0;
+#pragma unroll
+    for (int k = 0; k < G::ROWS; ++k) {
+        const IDX row = row0 + k;
+        if (row >= nrows)
+            break;
+        const int Y = (int)(row % (IDX)L.rows);
+        const IDX fz = row / (IDX)L.rows;
+        const int z = (int)(fz % (IDX)L.nz), f = (int)(fz / (IDX)L.nz);
+        int y = Y - GY;  // ny >= 8 > GY: one wrap is enough
+        y = y < 0 ? y + L.ny : (y >= L.ny ? y - L.ny : y);
+        s[k] = src + (((long long)f * L.nz + z) * L.ny + y) * L.nx;
+        d[k] = dst + (long long)f * L.fpitch + (long long)z * L.plane + (long long)Y * L.P;
+        n = k + 1;
+    }
     if (VEC) {
-        for (int x = 4 * lane; x < L.nx; x += 4 * 32) {
-            const Quad<TSrc> q = load_quad(s + x);
-            const TD v[4] = {(TD)q.v[0], (TD)q.v[1], (TD)q.v[2], (TD)q.v[3]};
-            store_quad(d + GX + x, v);
+        for (int x = 4 * lane; x < L.nx; x += 4 * LPR) {
+            Quad<TSrc> q[G::ROWS];
+#pragma unroll
+            for (int k = 0; k < G::ROWS; ++k)
+                if (k < n)
+                    q[k] = load_quad(s[k] + x);
+#pragma unroll
+            for (int k = 0; k < G::ROWS; ++k)
+                if (k < n) {
+                    const TD v[4] = {(TD)q[k].v[0], (TD)q[k].v[1], (TD)q[k].v[2], (TD)q[k].v[3]};
+                    store_quad(d[k] + GX + x, v);
+                    if (x == 0)
+                        store_quad(d[k] + GX + L.nx, v);
+                    if (x == L.nx - 4)
+                        store_quad(d[k], v);
+                }
         }
     } else {
-        for (int x = lane; x < L.nx; x += 32)
-            d[GX + x] = (TD)s[x];
-    }
-    if (lane < 2 * GX) {
-        const int X = lane < GX ? lane : L.nx + lane;
-        d[X] = (TD)s[wrapi(X - GX, L.nx)];
+#pragma unroll
+        for (int k = 0; k < G::ROWS; ++k)
+            if (k < n)
+                for (int X = lane; X < L.nx + 2 * GX; X += LPR)
+                    d[k][X] = (TD)s[k][wrapi(X - GX, L.nx)];
     }
 }
 
-// Interior rows back to the compact layout; one warp per row.
-template <class TS, class TD, bool VEC>
-__global__ void __launch_bounds__(32 * COPY_WARPS) k_gather(const TS *__restrict__ src,
-                                                           TD *__restrict__ dst, Layout L,
-                                                           long long nrows)
+// Interior rows back to the compact layout, in the same way.
+template <class TS, class TD, bool VEC, int LPR, class IDX>
+__global__ void __launch_bounds__(COPY_THREADS) k_gather(const TS *__restrict__ src,
+                                                        TD *__restrict__ dst, Layout L, IDX nrows)
 {
-    const long long row = (long long)blockIdx.x * COPY_WARPS + threadIdx.x / 32;
-    const int lane = threadIdx.x % 32;
-    if (row >= nrows)
-        return;
-    const int y = (int)(row % L.ny);
-    const long long fz = row / L.ny;
-    const int z = (int)(fz % L.nz), f = (int)(fz / L.nz);
-    const TS *s = src + lidx(L, f, z, y, 0);
-    TD *d = dst + row * L.nx;
+    using G = RowGroup<LPR>;
+    const int lane = threadIdx.x % LPR;
+    const IDX row0 = (IDX)blockIdx.x * G::PER_BLOCK + threadIdx.x / LPR * G::ROWS;
+    const TS *s[G::ROWS];
+    int n = 0;
+#pragma unroll
+    for (int k = 0; k < G::ROWS; ++k) {
+        const IDX row = row0 + k;
+        if (row >= nrows)
+            break;
+        const int y = (int)(row % (IDX)L.ny);
+        const IDX fz = row / (IDX)L.ny;
+        s[k] = src + lidx(L, (int)(fz / (IDX)L.nz), (int)(fz % (IDX)L.nz), y, 0);
+        n = k + 1;
+    }
+    TD *d = dst + (long long)row0 * L.nx;
     if (VEC) {
-        for (int x = 4 * lane; x < L.nx; x += 4 * 32) {
-            const Quad<TS> q = load_quad(s + x);
-            const TD v[4] = {(TD)q.v[0], (TD)q.v[1], (TD)q.v[2], (TD)q.v[3]};
-            store_quad(d + x, v);
+        for (int x = 4 * lane; x < L.nx; x += 4 * LPR) {
+            Quad<TS> q[G::ROWS];
+#pragma unroll
+            for (int k = 0; k < G::ROWS; ++k)
+                if (k < n)
+                    q[k] = load_quad(s[k] + x);
+#pragma unroll
+            for (int k = 0; k < G::ROWS; ++k)
+                if (k < n) {
+                    const TD v[4] = {(TD)q[k].v[0], (TD)q[k].v[1], (TD)q[k].v[2], (TD)q[k].v[3]};
+                    store_quad(d + (long long)k * L.nx + x, v);
+                }
         }
     } else {
-        for (int x = lane; x < L.nx; x += 32)
-            d[x] = (TD)s[x];
+#pragma unroll
+        for (int k = 0; k < G::ROWS; ++k)
+            if (k < n)
+                for (int x = lane; x < L.nx; x += LPR)
+                    d[(long long)k * L.nx + x] = (TD)s[k][x];
     }
 }
 
@@ -127,28 +176,52 @@ inline bool quad_ok(const void *compact, int nx)
     return ((uintptr_t)compact % 16) == 0 && nx % 4 == 0;
 }
 
+template <class TD, class TSrc, bool VEC, int LPR>
+cudaError_t scatter_r(const TSrc *src, TD *dst, const Layout &L, int nf, cudaStream_t stream)
+{
+    const long long nrows = (long long)nf * L.nz * L.rows, per = RowGroup<LPR>::PER_BLOCK;
+    const unsigned grid = (unsigned)((nrows + per - 1) / per);
+    if (nrows < (1LL << 31))
+        k_scatter<TD, TSrc, VEC, LPR, unsigned><<<grid, COPY_THREADS, 0, stream>>>(src, dst, L,
+                                                                                (unsigned)nrows);
+    else
+        k_scatter<TD, TSrc, VEC, LPR, unsigned long long><<<grid, COPY_THREADS, 0, stream>>>(
+            src, dst, L, (unsigned long long)nrows);
+    return cudaGetLastError();
+}
+
 template <class TD, class TSrc>
 cudaError_t scatter_t(const TSrc *src, TD *dst, const Layout &L, int nf, cudaStream_t stream)
 {
-    const long long nrows = (long long)nf * L.nz * L.rows;
-    const dim3 grid((unsigned)((nrows + COPY_WARPS - 1) / COPY_WARPS)), block(32 * COPY_WARPS);
-    if (quad_ok(src, L.nx))
-        k_scatter<TD, TSrc, true><<<grid, block, 0, stream>>>(src, dst, L, nrows);
+    if (!quad_ok(src, L.nx))
+        return scatter_r<TD, TSrc, false, 32>(src, dst, L, nf, stream);
+    return L.nx <= 32   ? scatter_r<TD, TSrc, true, 8>(src, dst, L, nf, stream)
+           : L.nx <= 64 ? scatter_r<TD, TSrc, true, 16>(src, dst, L, nf, stream)
+                        : scatter_r<TD, TSrc, true, 32>(src, dst, L, nf, stream);
+}
+
+template <class TS, class TD, bool VEC, int LPR>
+cudaError_t gather_r(const TS *src, TD *dst, const Layout &L, int nf, cudaStream_t stream)
+{
+    const long long nrows = (long long)nf * L.nz * L.ny, per = RowGroup<LPR>::PER_BLOCK;
+    const unsigned grid = (unsigned)((nrows + per - 1) / per);
+    if (nrows < (1LL << 31))
+        k_gather<TS, TD, VEC, LPR, unsigned><<<grid, COPY_THREADS, 0, stream>>>(src, dst, L,
+                                                                             (unsigned)nrows);
     else
-        k_scatter<TD, TSrc, false><<<grid, block, 0, stream>>>(src, dst, L, nrows);
+        k_gather<TS, TD, VEC, LPR, unsigned long long><<<grid, COPY_THREADS, 0, stream>>>(
+            src, dst, L, (unsigned long long)nrows);
     return cudaGetLastError();
 }
 
 template <class TS, class TD>
 cudaError_t gather_t(const TS *src, TD *dst, const Layout &L, int nf, cudaStream_t stream)
 {
-    const long long nrows = (long long)nf * L.nz * L.ny;
-    const dim3 grid((unsigned)((nrows + COPY_WARPS - 1) / COPY_WARPS)), block(32 * COPY_WARPS);
-    if (quad_ok(dst, L.nx))
-        k_gather<TS, TD, true><<<grid, block, 0, stream>>>(src, dst, L, nrows);
-    else
-        k_gather<TS, TD, false><<<grid, block, 0, stream>>>(src, dst, L, nrows);
-    return cudaGetLastError();
+    if (!quad_ok(dst, L.nx))
+        return gather_r<TS, TD, false, 32>(src, dst, L, nf, stream);
+    return L.nx <= 32   ? gather_r<TS, TD, true, 8>(src, dst, L, nf, stream)
+           : L.nx <= 64 ? gather_r<TS, TD, true, 16>(src, dst, L, nf, stream)
+                        : gather_r<TS, TD, true, 32>(src, dst, L, nf, stream);
 }
 
 // ------------------------------------------------------ ghost planes in z
