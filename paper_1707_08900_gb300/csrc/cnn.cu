@@ -7,12 +7,12 @@
 //   N = the output channels of the three z taps of one (dy, dx) tap (they
 //   share the A window), K = 9 (dy, dx) taps x input channels; BF16 operands
 //   in shared memory as K-major core matrices, FP32 accumulators in TMEM.
-// * A persistent, warp-specialised CTA per SM: one warp loads each tile's
-//   input plus its periodic one-point halo with ONE TMA box into a two- or
-//   three-stage ring, one thread issues the tile's MMAs from shifted
-//   descriptors into one of two TMEM accumulator buffers, and eight
-//   epilogue warps read the other buffer (bias, GELU or GELU', BF16 stores),
-//   so loads, MMAs and epilogues of consecutive tiles overlap.  The weights
+// * A persistent, warp-specialised CTA per SM streams columns of the grid along
+//   z: one warp loads each plane plus its periodic one-point halo with ONE TMA
+//   box into a ring of stages, one thread issues the plane's MMAs from shifted
+//   descriptors into a ring of TMEM accumulators (one per output plane), and
+//   sixteen epilogue warps drain finished planes (bias, GELU or GELU', BF16
+//   stores), so loads, MMAs and epilogues of neighbouring planes overlap.  The weights
 //   (B operand) stay in shared memory.  Activations are kept in a padded,
 //   chunk-major layout whose one-point frame holds the periodic copies, so a
 //   halo never wraps.  The input gradient is the same kernel with the
@@ -82,12 +82,44 @@ __host__ __device__ inline int core_idx(int n, int k, int K)
     return (n / 8) * (K * 8) + (k / 8) * 64 + (n % 8) * 8 + (k % 8);
 }
 
-__device__ __forceinline__ float gelu(float h) { return 0.5f * h * (1.0f + erff(h * 0.70710678118654752f)); }
-
-__device__ __forceinline__ float gelu_grad(float h)
+// Exact GELU h Phi(h) and its derivative Phi(h) + h phi(h), two values at a time
+// in packed FP32x2 arithmetic.  With x = |h| and t = 1 / (1 + p x),
+//   1 - Phi(x) = exp(-x^2 / 2) t P(t),
+// P a degree-7 polynomial fitted here to the complementary error function
+// (minimax in relative error over 0 <= x <= 13.5, p chosen with it: 1.1e-7).
+// In FP32, max |error| of GELU over |h| <= 9 is 3.8e-7 (4.5e-7 by erff) and the
+// negative tail keeps its relative accuracy (1e-6 at h > -4, 5e-4 by 1 + erff).
+// About 13 instructions per value where erff and the rest take 45: the
+// epilogues' issue slots bound the convolutions together with the MMAs.
+struct Phi2 {
+    float2 phi, dens;  // Phi(h), exp(-h^2 / 2)
+};
+__device__ __forceinline__ Phi2 phi2(const float2 h)
 {
-    return 0.5f * (1.0f + erff(h * 0.70710678118654752f)) +
-           h * expf(-0.5f * h * h) * 0.39894228040143268f;
+    const float2 x = make_float2(fabsf(h.x), fabsf(h.y));
+    auto bc = [](float v) { return make_float2(v, v); };
+    const float2 den = __ffma2_rn(bc(0.235f), x, bc(1.f));
+    const float2 t = make_float2(__fdividef(1.f, den.x), __fdividef(1.f, den.y));
+    const float2 a = __fmul2_rn(__fmul2_rn(x, x), bc(-0.72134752f));  // log2(e) / 2
+    Phi2 r;
+    r.dens = make_float2(exp2f(a.x), exp2f(a.y));
+    float2 p = bc(-0.0640975162f);
+    p = __ffma2_rn(p, t, bc(0.209975779f));
+    p = __ffma2_rn(p, t, bc(-0.145442292f));
+    p = __ffma2_rn(p, t, bc(0.179566205f));
+    p = __ffma2_rn(p, t, bc(0.0356354676f));
+    p = __ffma2_rn(p, t, bc(0.0979318768f));
+    p = __ffma2_rn(p, t, bc(0.0926214978f));
+    p = __ffma2_rn(p, t, bc(0.0938089192f));
+    const float2 q = __fmul2_rn(r.dens, __fmul2_rn(p, t));
+    r.phi = make_float2(h.x >= 0.f ? 1.f - q.x : q.x, h.y >= 0.f ? 1.f - q.y : q.y);
+    return r;
+}
+__device__ __forceinline__ float2 gelu2(const float2 h) { return __fmul2_rn(h, phi2(h).phi); }
+__device__ __forceinline__ float2 gelu_grad2(const float2 h)
+{
+    const Phi2 r = phi2(h);
+    return __ffma2_rn(__fmul2_rn(h, make_float2(0.39894228f, 0.39894228f)), r.dens, r.phi);
 }
 
 // Activations live in a padded, chunk-major layout: act[c8][b][zp][yp][xp][8]
@@ -122,52 +154,55 @@ __device__ __forceinline__ void each_copy(int x, int y, int z, int n, F &&f)
 struct ConvArgs {
     const bf16 *wB;      // [N][27*CIN] in core-matrix order
     const float *bias;   // [N]                      (EPI_GELU, EPI_LINEAR)
-    float *hsave;        // [npts][N] pre-activation (EPI_GELU; NULL: not kept)
+    float4 *hsave;       // pre-activation (EPI_GELU; NULL: not kept), [N/4][B n^3] quads
     bf16 *yb;            // padded chunk-major output (EPI_GELU: GELU(h), EPI_DGELU: dh)
     float *yf;           // [npts][8]                (EPI_LINEAR)
-    const float *hprev;  // [npts][N]                (EPI_DGELU)
+    const float4 *hprev; // the same quads           (EPI_DGELU)
     int n;               // grid side
     int npts;            // batch * n^3
     int B;               // samples allocated in the padded arrays
+    int run;             // output planes of a run (conv_run)
     int *dev_error;
 };
 
-// A conv tile is TXT x TYT points in each of ZB consecutive z planes: one
-// M = 128 MMA row block per plane, row r = point (x0 + r % TXT, y0 + r / TXT).
-// Its input plus the one-point halo, HX x HY x HZ points of CIN channels, is
-// ONE TMA box of the padded chunk-major input, (8 channels, HX, HY, HZ,
-// CIN / 8 chunks): in shared memory chunk c of halo point (hx, hy, hz) sits at
-// c * CS + ((hz * HY + hy) * HX + hx) * 16.  The A operand of halo plane hz
-// and in-plane tap (dy, dx) is that buffer at a shifted start: core matrices
-// of 8 x-consecutive rows (16-byte row stride), row groups one halo row apart
-// (SBO = HX * 16), K chunks CS apart (LBO).
+// A conv column is TXT x TYT points of every z plane of a sample: one M = 128
+// MMA row block per plane, row r = point (x0 + r % TXT, y0 + r / TXT).  A plane
+// of its input plus the one-point halo, HX x HY points of CIN channels, is ONE
+// TMA box of the padded chunk-major input, (8 channels, HX, HY, 1, CIN / 8
+// chunks): in shared memory chunk c of halo point (hx, hy) sits at
+// c * CS + (hy * HX + hx) * 16.  The A operand of in-plane tap (dy, dx) is that
+// buffer at a shifted start: core matrices of 8 x-consecutive rows (16-byte row
+// stride), row groups one halo row apart (SBO = HX * 16), K chunks CS apart
+// (LBO).
 //
-// The three z taps of one (dy, dx) read the same A window (halo plane hz
-// feeds output planes hz - dz for dz = 0, 1, 2), so they are ONE MMA with
-// their weights stacked along N (N = 3 NO for NO output channels): a
-// tcgen05 MMA of M = 128, K = 16 costs about the same for N = 16 or 32 as for
-// 96 (measured on GB300: 45 cycles for N <= 32, 56 for N = 96, 64 for 128),
-// so merging the z taps cuts the MMA time per output plane by about 2.4 at
-// ZB = 4.  Column group dz of the MMA of halo plane hz lands on output plane
-// zo = hz - dz; placing plane zo's accumulator at column NO (ZB + 1 - zo)
-// makes the three groups of every MMA consecutive columns at
-// NO (ZB + 1 - hz).  Planes -2, -1, ZB and ZB + 1 catch the groups that fall
-// outside the tile (never read).  Every MMA accumulates, so the buffers
-// start at zero and the epilogue zeroes the columns it has read before
-// handing the buffer back.
-constexpr int TXT = 8, TYT = 16, ZB = 4;
-constexpr int HX = TXT + 2, HY = TYT + 2, HZ = ZB + 2, HPTS = HX * HY * HZ;
-static_assert(TXT * TYT == MT, "one MMA row block per tile plane");
+// The three z taps of one (dy, dx) read the same A window (input plane j, j = 0
+// one below the first output plane, feeds output planes j - dz for dz = 0, 1,
+// 2), so they are ONE MMA with their weights stacked along N (N = 3 NO for NO
+// output channels): a tcgen05 MMA of M = 128, K = 16 costs about the same for
+// N = 16 or 32 as for 96 (measured on GB300: 45 cycles for N <= 32, 56 for
+// N = 96, 64 for 128).  The accumulators of the output planes form a ring of
+// RING slots in TMEM, slot s at column NO (RING - 1 - s), so that planes j, j - 1
+// and j - 2 are consecutive columns; an MMA is cut in two where the ring wraps
+// and loses the groups outside the column at its ends.  Every MMA accumulates,
+// so the ring starts at zero and the epilogue zeroes the columns it has read.
+//
+// Streaming reads and multiplies every input plane once per run of output
+// planes (plus two at its ends); four-plane tiles with their own halo took six
+// planes for four.
+constexpr int TXT = 8, TYT = 16;
+constexpr int HX = TXT + 2, HY = TYT + 2, HPTS = HX * HY;
+static_assert(TXT * TYT == MT, "one MMA row block per plane");
 constexpr int TAPS_XY = 9;  // (dy, dx) taps; dz is stacked along N
 
-// Warp roles of the convolution CTA (one per SM, persistent over tiles):
-// warp 0 issues the TMA halo loads, warp 1 the MMAs (and owns the TMEM
-// allocation), warps 2-9 are the epilogue (warp w reads TMEM lanes
-// 32 (w % 4) .. 32 (w % 4) + 31; warps 2-5 the first half of the output
-// channels, 6-9 the second).
-constexpr int CONV_THREADS = 320;
-constexpr int EPI_WARPS = 8;
-constexpr int NACC = 2;  // TMEM accumulator buffers
+// Warp roles of the convolution CTA (one per SM, persistent): warp 0 issues the
+// TMA loads, warp 1 the MMAs (and owns the TMEM allocation), warps 2-17 are the
+// epilogue: two groups of eight take the planes in turn, so that one plane's
+// waits and stores overlap the next one's arithmetic (with one group every plane
+// paid its whole latency).  Warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31;
+// the first four warps of a group take the first half of the output channels.
+constexpr int EPI_WARPS = 8, EPI_GROUPS = 2;
+constexpr int CONV_THREADS = 32 * (2 + EPI_WARPS * EPI_GROUPS);
+constexpr int RING = 16;  // accumulator slots (output planes)
 
 template <int CIN, int NO, int EPI>
 struct ConvSmem {
@@ -177,31 +212,30 @@ struct ConvSmem {
     static constexpr int B_BYTES = N * K * 2;
     static constexpr int CS = HPTS * 16;  // chunk stride of the TMA box
     static constexpr int A_BYTES = CH8 * CS;
-    static constexpr int NSTAGE = CIN >= 32 ? 2 : 3;  // halo buffers
+    static constexpr int NSTAGE = CIN >= 32 ? 10 : 16;  // input planes in flight
     static constexpr int A_OFF = (B_BYTES + 1023) / 1024 * 1024;
-    static constexpr int A_PITCH = (A_BYTES + 1023) / 1024 * 1024;
+    static constexpr int A_PITCH = (A_BYTES + 127) / 128 * 128;
     static constexpr int BAR_OFF = A_OFF + NSTAGE * A_PITCH;
-    // full[NSTAGE], empty[NSTAGE], acc_full[NACC], acc_empty[NACC], then the
-    // TMEM address, the abort flag and four issue / consume counts
-    static constexpr int BYTES = BAR_OFF + (2 * NSTAGE + 2 * NACC) * 8 + 8 + 16;
-    static constexpr int ACC_COLS = (ZB + 4) * NO;  // one accumulator buffer
-    static constexpr int TCOLS = NACC * ACC_COLS <= 128 ? 128 : (NACC * ACC_COLS <= 256 ? 256 : 512);
-    static_assert(NACC * ACC_COLS <= 512, "TMEM columns");
+    // full[NSTAGE], empty[NSTAGE], acc_full[RING], acc_empty[RING], stopped,
+    // then the TMEM address, the abort flag, six counts, the biases
+    static constexpr int BIAS_OFF = BAR_OFF + (2 * NSTAGE + 2 * RING + 1) * 8 + 8 + 24;
+    static constexpr int BYTES = BIAS_OFF + NO * 4;
+    static constexpr int TCOLS = RING * NO;
+    static_assert(TCOLS == 256 || TCOLS == 512, "TMEM columns");
     static_assert(CS % 16 == 0 && (CS >> 4) < (1 << 14) && ((K * 16) >> 4) < (1 << 14),
                   "descriptor offsets");
-    static_assert(BYTES <= 227 * 1024, "shared memory");
+    static_assert(BAR_OFF % 8 == 0 && BYTES <= 227 * 1024, "shared memory");
 };
 
-// Zeroes 16 (or 8) consecutive FP32 columns of this warp's 32 TMEM lanes and
-// waits for the stores to complete.
+// Zeroes 16 (or 8) consecutive FP32 columns of this warp's 32 TMEM lanes; the
+// stores are complete after wait_st().
 __device__ __forceinline__ void tmem_zero16(uint32_t taddr)
 {
     const uint32_t z = 0;
     __syncwarp();
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};\n\t"
-        "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+        "{%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
         "r"(z)
         : "memory");
 }
@@ -211,10 +245,15 @@ __device__ __forceinline__ void tmem_zero8(uint32_t taddr)
     const uint32_t z = 0;
     __syncwarp();
     asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};\n\t"
-        "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
         "r"(z)
         : "memory");
+}
+
+__device__ __forceinline__ void wait_st()
+{
+    __syncwarp();
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
@@ -242,16 +281,25 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, vo
     }
 }
 
-__device__ __forceinline__ void tile_origin(int tile, int n, int &x0, int &y0, int &z0, int &b)
+// The CTA's runs of up to `run` output planes along z inside one column:
+// f(x0, y0, sample, z0, planes) for each.  Every role walks them the same way.
+// CTAs that work at the same time take neighbouring columns at the same height,
+// so that the halo rows and the 128-byte rows they share meet in L2.
+template <class F>
+__device__ __forceinline__ void each_run(int n, int nb, int run, F &&f)
 {
-    const int tx_n = (n + TXT - 1) / TXT, ty_n = (n + TYT - 1) / TYT, tz_n = (n + ZB - 1) / ZB;
-    int r = tile;
-    x0 = (r % tx_n) * TXT;
-    r /= tx_n;
-    y0 = (r % ty_n) * TYT;
-    r /= ty_n;
-    z0 = (r % tz_n) * ZB;
-    b = r / tz_n;
+    const int tx_n = (n + TXT - 1) / TXT, ty_n = (n + TYT - 1) / TYT, tz_n = (n + run - 1) / run;
+    const int units = nb * tz_n * ty_n * tx_n;
+    for (int u = blockIdx.x; u < units; u += gridDim.x) {
+        int r = u;
+        const int x0 = (r % tx_n) * TXT;
+        r /= tx_n;
+        const int y0 = (r % ty_n) * TYT;
+        r /= ty_n;
+        const int z0 = (r % tz_n) * run;
+        if (!f(x0, y0, r / tz_n, z0, min(run, n - z0)))
+            return;
+    }
 }
 
 template <int CIN, int NO, int EPI>
@@ -260,7 +308,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
 {
     using SM = ConvSmem<CIN, NO, EPI>;
     constexpr int NSTAGE = SM::NSTAGE;
-    constexpr int KSTEPS = CIN / 16;  // MMAs per (dy, dx) tap and halo plane
+    constexpr int KSTEPS = CIN / 16;  // MMAs per (dy, dx) tap and input plane
     constexpr int SBO_B = SM::K * 16;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *sB = smem;
@@ -268,10 +316,13 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + SM::BAR_OFF);
     uint64_t *empty = full + NSTAGE;
     uint64_t *accf = empty + NSTAGE;
-    uint64_t *acce = accf + NACC;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(acce + NACC);
+    uint64_t *acce = accf + RING;
+    uint64_t *stopped = acce + RING;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(stopped + 1);
     volatile int *abort = reinterpret_cast<volatile int *>(tslot + 1);
-    int *cnt = reinterpret_cast<int *>(tslot + 2);  // issued, consumed, committed, drained
+    // copies issued / waited for, planes committed, MMAs cut short, planes
+    // drained by each group
+    int *cnt = reinterpret_cast<int *>(tslot + 2);
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 
     // epilogue geometry: two warps per TMEM lane quarter, each taking half
@@ -279,7 +330,10 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     constexpr int NH = NO / 2;  // channels per epilogue warp
     static_assert(NH == 16 || NH == 8, "epilogue column chunks");
     const int e = warp - 2;
-    const int q = warp % 4, c0 = (e / 4) * NH;
+    const int group = e / EPI_WARPS;
+    const int q = warp % 4, c0 = (e % EPI_WARPS / 4) * NH;
+    float *sbias = reinterpret_cast<float *>(smem + SM::BIAS_OFF);
+    // zeroes NH columns of the warp's lanes; complete after wait_st()
     auto zero_cols = [&](uint32_t taddr) {
         if constexpr (NH == 16)
             tmem_zero16(taddr);
@@ -295,14 +349,18 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             tiled::mbar_init(&full[s], 1);
             tiled::mbar_init(&empty[s], 1);
         }
-        for (int s = 0; s < NACC; ++s) {
+        for (int s = 0; s < RING; ++s) {
             tiled::mbar_init(&accf[s], 1);
             tiled::mbar_init(&acce[s], EPI_WARPS);  // one arrival per epilogue warp
         }
+        tiled::mbar_init(stopped, 1);
         *abort = 0;
-        cnt[0] = cnt[1] = cnt[2] = cnt[3] = 0;
+        for (int i = 0; i < 6; ++i)
+            cnt[i] = 0;
         tiled::fence_mbar_init();
     }
+    if (EPI != EPI_DGELU && threadIdx.x < NO)
+        sbias[threadIdx.x] = a.bias[threadIdx.x];
     if (warp == 1)
         tc::tmem_alloc(tslot, SM::TCOLS);
     tc::fence_smem_to_async();  // the weights, written by the generic proxy, feed the MMAs
@@ -310,12 +368,13 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(tslot);
-    // every MMA accumulates: both accumulator buffers start at zero
+    // every MMA accumulates: the accumulators start at zero
     if (warp >= 2) {
         const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + c0;
 #pragma unroll 1
-        for (int j = 0; j < NACC * (ZB + 4); ++j)
+        for (int j = group; j < RING; j += EPI_GROUPS)
             zero_cols(tl + j * NO);
+        wait_st();
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -329,168 +388,231 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     const int n = a.n;
     const long long n3 = (long long)n * n * n;
     const int nb = (int)(a.npts / n3);
-    const int ntiles = nb * ((n + ZB - 1) / ZB) * ((n + TYT - 1) / TYT) * ((n + TXT - 1) / TXT);
 
     if (warp == 0) {
-        // producer: one halo box per tile into the stage the MMAs freed
+        // producer: one haloed plane per stage the MMAs freed
         if (lane == 0) {
             int i = 0;
-            for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
-                const int s = i % NSTAGE;
-                if (!wait_or_abort(&empty[s], ((i / NSTAGE) & 1) ^ 1, abort))
-                    break;
-                int x0, y0, z0, b;
-                tile_origin(tile, n, x0, y0, z0, b);
-                tiled::mbar_expect_tx(&full[s], SM::A_BYTES);
-                // padded coordinates of the halo's first point: (x0 - 1) + 1;
-                // x and the 8 channels of a chunk form one 160-byte row
-                tiled::tma_load_4d(sA + s * SM::A_PITCH, &xmap, &full[s], 8 * x0, y0,
-                                   b * (n + 2) + z0, 0);
-                cnt[0] = i + 1;
-            }
+            each_run(n, nb, a.run, [&](int x0, int y0, int b, int z0, int m) {
+                for (int j = 0; j < m + 2; ++j, ++i) {
+                    const int s = i % NSTAGE;
+                    if (!wait_or_abort(&empty[s], ((i / NSTAGE) & 1) ^ 1, abort))
+                        return false;
+                    tiled::mbar_expect_tx(&full[s], SM::A_BYTES);
+                    // padded coordinates of the halo's first point: (x0 - 1) +
+                    // 1; x and the 8 channels of a chunk form one 160-byte row
+                    tiled::tma_load_4d(sA + s * SM::A_PITCH, &xmap, &full[s], 8 * x0, y0,
+                                       b * (n + 2) + z0 + j, 0);
+                    cnt[0] = i + 1;
+                }
+                return true;
+            });
         }
     } else if (warp == 1) {
-        // MMA issuer: per halo plane, 9 (dy, dx) taps x KSTEPS MMAs of
-        // N = 3 NO into one of two accumulator buffers; the commits free the
-        // halo stage and hand the accumulators to the epilogue
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(MT, SM::N);
-            // descriptors of the stage and weight bases; every tap's operand
-            // is a compile-time byte offset from them (the start address is
-            // the descriptor's low field, in 16-byte units, and shared
-            // memory addresses stay below 2^18 bytes, so adding the offset
-            // cannot carry into the next field)
-            const uint64_t bd0 = tc::smem_desc(tc::smem_u32(sB), 128, SBO_B);
-            const uint64_t ad0 = tc::smem_desc(tc::smem_u32(sA), SM::CS, HX * 16);
-            int i = 0;
-            for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
-                const int s = i % NSTAGE, acc = i % NACC;
-                if (!wait_or_abort(&full[s], (i / NSTAGE) & 1, abort))
-                    break;
+        // MMA issuer: per input plane, 9 (dy, dx) taps x KSTEPS MMAs of up to
+        // 3 NO columns; the commits free the stage and hand finished output
+        // planes to the epilogue.  The whole warp runs the loop, one lane issues
+        // (tc::mma_bf16_elect)
+        const uint32_t elected = tc::elect_one();
+        // descriptors of the stage and weight bases; every tap's operand
+        // is a compile-time byte offset from them (the start address is
+        // the descriptor's low field, in 16-byte units, and shared
+        // memory addresses stay below 2^18 bytes, so adding the offset
+        // cannot carry into the next field)
+        const uint64_t bd0 = tc::smem_desc(tc::smem_u32(sB), 128, SBO_B);
+        const uint64_t ad0 = tc::smem_desc(tc::smem_u32(sA), SM::CS, HX * 16);
+        // CNT z taps from dz0 on, into consecutive slots down from `slot`
+        auto issue = [&](uint64_t ad, int slot, int dz0, auto cntc) {
+            constexpr uint32_t idesc = tc::idesc_bf16_f32(MT, decltype(cntc)::value * NO);
+            const uint64_t bd = bd0 + (uint64_t)(dz0 * (NO / 8) * (SBO_B >> 4));
+            const uint32_t d = tmem + (uint32_t)(NO * (RING - 1 - slot));
+#pragma unroll
+            for (int t = 0; t < TAPS_XY; ++t)
+#pragma unroll
+                for (int k = 0; k < KSTEPS; ++k)
+                    tc::mma_bf16_elect(
+                        elected, d,
+                        ad + (uint64_t)((((t / 3) * HX + t % 3) * 16 + 2 * k * SM::CS) >> 4),
+                        bd + (uint64_t)((t * KSTEPS + k) * 16), idesc, 1u);
+        };
+        auto issue_n = [&](uint64_t ad, int slot, int dz0, int cnt_z) {
+            if (cnt_z == 3)
+                issue(ad, slot, 0, std::integral_constant<int, 3>{});
+            else if (cnt_z == 2)
+                issue(ad, slot, dz0, std::integral_constant<int, 2>{});
+            else
+                issue(ad, slot, dz0, std::integral_constant<int, 1>{});
+        };
+        int i = 0, done = 0;  // planes loaded, output planes of earlier runs
+        bool ok = true;
+        auto wait = [&](uint64_t *bar, int phase) {
+            ok = __all_sync(0xffffffffu, wait_or_abort(bar, phase, abort));
+            return ok;
+        };
+        each_run(n, nb, a.run, [&](int, int, int, int, int m) {
+#pragma unroll 1
+            for (int j = 0; j < m + 2; ++j, ++i) {
+                const int s = i % NSTAGE;
+                if (!wait(&full[s], (i / NSTAGE) & 1))
+                    return false;
                 cnt[1] = i + 1;
-                if (!wait_or_abort(&acce[acc], ((i / NACC) & 1) ^ 1, abort))
-                    break;
+                if (j < m) {  // output plane j begins: its slot must be drained and zero
+                    const int o = done + j;
+                    if (!wait(&acce[o % RING], ((o / RING) & 1) ^ 1))
+                        return false;
+                }
                 tc::fence_after_sync();
-                const uint64_t adst = ad0 + (uint64_t)((s * SM::A_PITCH) >> 4);
-                const uint32_t dbuf = tmem + acc * SM::ACC_COLS;
-#pragma unroll
-                for (int hz = 0; hz < HZ; ++hz)
-#pragma unroll
-                    for (int t = 0; t < TAPS_XY; ++t) {
-                        const int dy = t / 3, dx = t % 3;  // offset + 1
-#pragma unroll
-                        for (int k = 0; k < KSTEPS; ++k) {
-                            const int aoff =
-                                (((hz * HY + dy) * HX + dx) * 16 + 2 * k * SM::CS) >> 4;
-                            tc::mma_bf16(dbuf + (uint32_t)(NO * (ZB + 1 - hz)),
-                                         adst + (uint64_t)aoff,
-                                         bd0 + (uint64_t)((t * KSTEPS + k) * 16), idesc, 1u);
-                        }
-                    }
-                tc::commit(&empty[s]);
-                tc::commit(&accf[acc]);
-                cnt[2] = i + 1;
+                const uint64_t ad = ad0 + (uint64_t)((s * SM::A_PITCH) >> 4);
+                // z taps whose output plane j - dz lies in the run, cut
+                // where the slots wrap
+                const int lo = max(0, j - m + 1), hi = min(2, j);
+                const int slot = (done + j - lo) % RING;
+                const int first = min(hi - lo + 1, slot + 1);
+                issue_n(ad, slot, lo, first);
+                if (first < hi - lo + 1)
+                    issue_n(ad, RING - 1, lo + first, hi - lo + 1 - first);
+                tc::commit_elect(elected, &empty[s]);
+                if (j >= 2) {
+                    tc::commit_elect(elected, &accf[(done + j - 2) % RING]);
+                    cnt[2] = done + j - 1;
+                }
             }
+            done += m;
+            return true;
+        });
+        if (!ok) {  // a wait gave up: the MMAs issued so far are waited for below
+            tc::commit_elect(elected, stopped);
+            cnt[3] = 1;
         }
     } else {
-        // epilogue, per tile plane: TMEM -> registers, zero those columns,
+        // epilogue, per output plane: TMEM -> registers, zero those columns,
         // then bias / GELU / GELU' and the stores (with the periodic copies)
         const int r = q * 32 + lane;  // row of the M block = TMEM lane
         const int lx = r % TXT, ly = r / TXT;
         const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + c0;
-        float bias[NH];
-#pragma unroll
-        for (int j = 0; j < NH; ++j)
-            bias[j] = (EPI == EPI_DGELU || c0 + j >= NO) ? 0.f : __ldg(a.bias + c0 + j);
-        int i = 0;
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++i) {
-            const int acc = i % NACC;
-            // one lane waits, the warp follows it (the TMEM accesses below
-            // are warp-collective)
-            int ok = 0;
-            if (lane == 0)
-                ok = wait_or_abort(&accf[acc], (i / NACC) & 1, abort);
-            if (!__shfl_sync(0xffffffffu, ok, 0))
-                break;
-            // the other lanes observe the completed phase too (it cannot
-            // move on before this warp releases the buffer)
-            if (lane != 0)
-                (void)tiled::mbar_try_wait(&accf[acc], (i / NACC) & 1);
-            tc::fence_after_sync();
-            const uint32_t tb = tl + acc * SM::ACC_COLS;
-            int x0, y0, z0, b;
-            tile_origin(tile, n, x0, y0, z0, b);
+        const long long hq = (long long)a.B * n3;  // quads per channel group of h
+        const long long m2 = (long long)(n + 2) * (n + 2), yc = m2 * (n + 2) * a.B;
+        uint4 *yb = reinterpret_cast<uint4 *>(a.yb);
+        int o0 = 0;  // output planes of earlier runs
+        each_run(n, nb, a.run, [&](int x0, int y0, int b, int z0, int m) {
             const int x = x0 + lx, y = y0 + ly;
+            const bool inside = x < n && y < n;
+            // the point's chunk in the padded output, plane 0 of the frame, and
+            // the offsets of its periodic copies in x and y (0: none)
+            const long long col = aidx(c0 / 8, b, 0, y + 1, x + 1, n, a.B);
+            const long long dx = x == 0 ? n : (x == n - 1 ? -n : 0);
+            const long long dy = (long long)(n + 2) * (y == 0 ? n : (y == n - 1 ? -n : 0));
 #pragma unroll 1
-            for (int zo = 0; zo < ZB; ++zo) {
-                const uint32_t tp = tb + (uint32_t)(NO * (ZB + 1 - zo));
+            for (int k = (group + o0) & 1; k < m; k += EPI_GROUPS) {
+                const int o = o0 + k, z = z0 + k, slot = o % RING;
+                const long long p = (long long)b * n3 + ((long long)z * n + y) * n + x;
+                // the saved pre-activations, on their way during the wait
+                float4 hv[EPI == EPI_DGELU ? NH / 4 : 1];
+                if constexpr (EPI == EPI_DGELU) {
+                    if (inside)
+#pragma unroll
+                        for (int c = 0; c < NH / 4; ++c)
+                            hv[c] = __ldg(a.hprev + (c0 / 4 + c) * hq + p);
+                }
+                // one lane waits, the warp follows it (the TMEM accesses below
+                // are warp-collective)
+                int ok = 0;
+                if (lane == 0)
+                    ok = wait_or_abort(&accf[slot], (o / RING) & 1, abort);
+                if (!__shfl_sync(0xffffffffu, ok, 0))
+                    return false;
+                // the other lanes observe the completed phase too (it cannot
+                // move on before this warp releases the slot)
+                if (lane != 0)
+                    (void)tiled::mbar_try_wait(&accf[slot], (o / RING) & 1);
+                tc::fence_after_sync();
+                const uint32_t tp = tl + (uint32_t)(NO * (RING - 1 - slot));
                 float v[NH];
                 if constexpr (NH == 16)
                     tc::tmem_ld16(tp, v);
                 else
                     tc::tmem_ld8(tp, v);
                 zero_cols(tp);
-                const int z = z0 + zo;
-                if (x >= n || y >= n || z >= n)
-                    continue;
-                const long long p = (long long)b * n3 + ((long long)z * n + y) * n + x;
-                if constexpr (EPI == EPI_LINEAR) {
-                    // five real output channels, all in the first half
-                    if (c0 == 0) {
-                        float4 *yo = reinterpret_cast<float4 *>(a.yf + p * 8);
-                        yo[0] = make_float4(v[0] + bias[0], v[1] + bias[1], v[2] + bias[2],
-                                            v[3] + bias[3]);
-                        yo[1] = make_float4(v[4] + bias[4], 0.f, 0.f, 0.f);
-                    }
-                } else {
-                    uint4 out[NH / 8];
-#pragma unroll
-                    for (int c = 0; c < NH; c += 8) {
-                        float h[8];
-                        if constexpr (EPI == EPI_GELU) {
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                h[j] = v[c + j] + bias[c + j];
-                            if (a.hsave) {
-                                float4 *hs = reinterpret_cast<float4 *>(a.hsave + p * NO + c0 + c);
-                                hs[0] = make_float4(h[0], h[1], h[2], h[3]);
-                                hs[1] = make_float4(h[4], h[5], h[6], h[7]);
-                            }
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                h[j] = gelu(h[j]);
-                        } else {
-                            const float4 *hp =
-                                reinterpret_cast<const float4 *>(a.hprev + p * NO + c0 + c);
-                            const float4 h0 = __ldg(hp), h1 = __ldg(hp + 1);
-                            const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                h[j] = v[c + j] * gelu_grad(hv[j]);
+                if (inside) {
+                    if constexpr (EPI == EPI_LINEAR) {
+                        // five real output channels, all in the first half
+                        if (c0 == 0) {
+                            float4 *yo = reinterpret_cast<float4 *>(a.yf + p * 8);
+                            yo[0] = make_float4(v[0] + sbias[0], v[1] + sbias[1], v[2] + sbias[2],
+                                                v[3] + sbias[3]);
+                            yo[1] = make_float4(v[4] + sbias[4], 0.f, 0.f, 0.f);
                         }
-                        __nv_bfloat162 o[4];
+                    } else {
+                        uint4 out[NH / 8];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            o[j] = __floats2bfloat162_rn(h[2 * j], h[2 * j + 1]);
-                        out[c / 8] = *reinterpret_cast<uint4 *>(o);
+                        for (int c = 0; c < NH; c += 8) {
+                            float2 h[4];
+                            if constexpr (EPI == EPI_GELU) {
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    h[j] = __fadd2_rn(
+                                        make_float2(v[c + 2 * j], v[c + 2 * j + 1]),
+                                        *reinterpret_cast<const float2 *>(sbias + c0 + c + 2 * j));
+                                if (a.hsave) {
+                                    float4 *hs = a.hsave + (c0 + c) / 4 * hq + p;
+                                    hs[0] = make_float4(h[0].x, h[0].y, h[1].x, h[1].y);
+                                    hs[hq] = make_float4(h[2].x, h[2].y, h[3].x, h[3].y);
+                                }
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    h[j] = gelu2(h[j]);
+                            } else {
+                                const float4 h0 = hv[c / 4], h1 = hv[c / 4 + 1];
+                                h[0] = gelu_grad2(make_float2(h0.x, h0.y));
+                                h[1] = gelu_grad2(make_float2(h0.z, h0.w));
+                                h[2] = gelu_grad2(make_float2(h1.x, h1.y));
+                                h[3] = gelu_grad2(make_float2(h1.z, h1.w));
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    h[j] = __fmul2_rn(make_float2(v[c + 2 * j], v[c + 2 * j + 1]),
+                                                      h[j]);
+                            }
+                            __nv_bfloat162 w[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                w[j] = __floats2bfloat162_rn(h[j].x, h[j].y);
+                            out[c / 8] = *reinterpret_cast<uint4 *>(w);
+                        }
+                        // the point and its periodic copies in x, y and z
+                        auto put = [&](long long i) {
+#pragma unroll
+                            for (int c = 0; c < NH / 8; ++c)
+                                yb[i + c * yc] = out[c];
+                        };
+                        auto put_xy = [&](long long i) {
+                            put(i);
+                            if (dx)
+                                put(i + dx);
+                            if (dy) {
+                                put(i + dy);
+                                if (dx)
+                                    put(i + dy + dx);
+                            }
+                        };
+                        put_xy(col + (z + 1) * m2);
+                        if (z == 0)
+                            put_xy(col + (n + 1) * m2);
+                        else if (z == n - 1)
+                            put_xy(col);
                     }
-                    uint4 *yb = reinterpret_cast<uint4 *>(a.yb);
-                    each_copy(x, y, z, n, [&](int xp, int yp, int zp) {
-#pragma unroll
-                        for (int k8 = 0; k8 < NH / 8; ++k8)
-                            yb[aidx(c0 / 8 + k8, b, zp, yp, xp, n, a.B)] = out[k8];
-                    });
                 }
+                // the zeroed columns go back to the MMAs
+                wait_st();
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0)
+                    mbar_arrive(&acce[slot]);
+                if (e % EPI_WARPS == 0 && lane == 0)
+                    cnt[4 + group] = o + 1;
             }
-            // (the spill planes -2, -1, ZB, ZB + 1 keep accumulating: they are
-            // never read, and their columns are no other plane's)
-            tc::fence_before_sync();
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(&acce[acc]);
-            if (e == 0 && lane == 0)
-                cnt[3] = i + 1;
-        }
+            o0 += m;
+            return true;
+        });
     }
     __syncthreads();
     if (*abort) {
@@ -501,8 +623,11 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             volatile int never = 0;
             for (int j = cnt[1]; j < cnt[0]; ++j)
                 (void)wait_or_abort(&full[j % NSTAGE], (j / NSTAGE) & 1, &never);
-            for (int j = cnt[3]; j < cnt[2]; ++j)
-                (void)wait_or_abort(&accf[j % NACC], (j / NACC) & 1, &never);
+            for (int j = min(cnt[4], cnt[5]); j < cnt[2]; ++j)
+                if (j >= cnt[4 + (j & 1)])
+                    (void)wait_or_abort(&accf[j % RING], (j / RING) & 1, &never);
+            if (cnt[3])
+                (void)wait_or_abort(stopped, 0, &never);
         }
         __syncthreads();
     }
@@ -519,25 +644,23 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
 namespace gbfd {
 namespace cnn {
 
-// Normalised BF16 input of layer 1 (C0 = 16 channels, zero beyond the nf
-// physical fields) at point (b, x, y, z) into the padded chunk-major x0,
-// with its periodic copies.
-__device__ __forceinline__ void put_input(bf16 *x0, const float *v, int b, int x, int y, int z,
-                                          int n, int B)
+// The 8 channels of chunk 0 of point (b, x, y, z) into a 16-channel padded
+// activation, with its periodic copies.  Channels 8 to 15 are padding that stays
+// zero from the network's creation on.
+__device__ __forceinline__ void put_chunk0(bf16 *dst, const float (&v)[8], int b, int x, int y, int z,
+                                           int n, int B)
 {
-    __nv_bfloat162 o[8];
+    __nv_bfloat162 o[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 4; ++i)
         o[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-    const uint4 c0 = reinterpret_cast<uint4 *>(o)[0], c1 = reinterpret_cast<uint4 *>(o)[1];
-    uint4 *dst = reinterpret_cast<uint4 *>(x0);
-    each_copy(x, y, z, n, [&](int xp, int yp, int zp) {
-        dst[aidx(0, b, zp, yp, xp, n, B)] = c0;
-        dst[aidx(1, b, zp, yp, xp, n, B)] = c1;
-    });
+    const uint4 c0 = *reinterpret_cast<uint4 *>(o);
+    uint4 *d = reinterpret_cast<uint4 *>(dst);
+    each_copy(x, y, z, n, [&](int xp, int yp, int zp) { d[aidx(0, b, zp, yp, xp, n, B)] = c0; });
 }
 
-// Layer-1 input from compact FP32 states [batch][5][n^3] (nf fields present).
+// Layer-1 input, normalised, from compact FP32 states [batch][5][n^3] (nf fields
+// present).
 __global__ void k_input_compact(const float *__restrict__ xs, int nf, int n, int npts, int B,
                                 const float *__restrict__ mean, const float *__restrict__ stdv,
                                 bf16 *__restrict__ x0)
@@ -548,11 +671,11 @@ __global__ void k_input_compact(const float *__restrict__ xs, int nf, int n, int
         return;
     const int n3 = n * n * n;
     const int b = p / n3, r = p - b * n3;
-    float v[C0];
+    float v[8];
 #pragma unroll
-    for (int c = 0; c < C0; ++c)
+    for (int c = 0; c < 8; ++c)
         v[c] = (c < nf) ? (xs[((long long)b * NC + c) * n3 + r] - mean[c]) / stdv[c] : 0.f;
-    put_input(x0, v, b, r % n, (r / n) % n, r / (n * n), n, B);
+    put_chunk0(x0, v, b, r % n, (r / n) % n, r / (n * n), n, B);
 }
 
 // Same from a solver context's padded FP32 state (one box, batch 1).
@@ -566,11 +689,11 @@ __global__ void k_input_state(const float *__restrict__ st, Layout L, int nf, in
     if (p >= n * n * n)
         return;
     const int z = p / (n * n), y = (p / n) % n, x = p % n;
-    float v[C0];
+    float v[8];
 #pragma unroll
-    for (int c = 0; c < C0; ++c)
+    for (int c = 0; c < 8; ++c)
         v[c] = (c < nf) ? (st[lidx(L, c, z, y, x)] - mean[c]) / stdv[c] : 0.f;
-    put_input(x0, v, 0, x, y, z, n, B);
+    put_chunk0(x0, v, 0, x, y, z, n, B);
 }
 
 // state += std_out * y (the de-normalised predicted residual), ghosts kept.
@@ -602,34 +725,50 @@ __global__ void k_output_compact(const float *__restrict__ y, int n3, int npts,
 }
 
 // MSE of the normalised residual: t = (target - x) / std_out; loss partial
-// sums per block (FP64) and dY3 = 2 (y - t) / count in BF16, channels-last.
-__global__ void k_loss(const float *__restrict__ y, const float *__restrict__ xs,
-                       const float *__restrict__ ts, const float *__restrict__ sout, int nf,
-                       int n, int npts, int B, float inv_count, bf16 *__restrict__ dy3,
-                       double *__restrict__ part)
+// sums per block (FP64) and dY3 = 2 (y - t) / count in BF16, channels-last.  A
+// thread takes LOSS_PTS points and sums their squares in float-float (products
+// and sums with their rounding errors, about 46 significant bits), one FP64 value
+// per thread: converting and adding every square in FP64 kept the narrow FP64
+// pipe busy for half of the kernel.
+constexpr int LOSS_PTS = 4;
+__global__ void __launch_bounds__(256) k_loss(const float *__restrict__ y, const float *__restrict__ xs,
+                                              const float *__restrict__ ts,
+                                              const float *__restrict__ sout, int nf, int n, int npts,
+                                              int B, float inv_count, bf16 *__restrict__ dy3,
+                                              double *__restrict__ part)
 {
     const int n3 = n * n * n;
     __shared__ double sh[256];
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (p < npts) {
-        const int b = p / n3, r = p - b * n3;
-        float d[C3];
+    float hi = 0.f, lo = 0.f;
 #pragma unroll
-        for (int c = 0; c < C3; ++c)
+    for (int k = 0; k < LOSS_PTS; ++k) {
+        const int p = (blockIdx.x * LOSS_PTS + k) * 256 + threadIdx.x;
+        if (p >= npts)
+            break;
+        const int b = p / n3, r = p - b * n3;
+        const float4 y4 = __ldg(reinterpret_cast<const float4 *>(y + (long long)p * 8));
+        const float yv[NC] = {y4.x, y4.y, y4.z, y4.w, __ldg(y + (long long)p * 8 + 4)};
+        float d[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
             d[c] = 0.f;
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             const long long i = ((long long)b * NC + c) * n3 + r;
             const float t = c < nf ? (ts[i] - xs[i]) / sout[c] : 0.f;
-            const float e = y[(long long)p * 8 + c] - t;
-            l += (double)e * (double)e;
+            const float e = yv[c] - t;
+            float sq, err, sum, rest;
+            two_prod(e, e, sq, err);
+            two_sum(hi, sq, sum, rest);
+            hi = sum;
+            lo = __fadd_rn(lo, __fadd_rn(rest, err));
             d[c] = 2.f * e * inv_count;
         }
         // dY3 into the padded chunk-major layout, with its periodic copies
-        put_input(dy3, d, b, r % n, (r / n) % n, r / (n * n), n, B);
+        put_chunk0(dy3, d, b, r % n, (r / n) % n, r / (n * n), n, B);
     }
-    sh[threadIdx.x] = l;
+    // (an overflowing or undefined sum has no error term)
+    sh[threadIdx.x] = isfinite(hi) ? (double)hi + (double)lo : (double)hi;
     __syncthreads();
     for (int s = 128; s > 0; s >>= 1) {
         if (threadIdx.x < s)
@@ -846,7 +985,8 @@ struct gbfd_cnn {
     float *bias[3];
     float *norm;  // mean_in[5], std_in[5], std_out[5]
     bf16 *x0, *a1, *a2, *dy3, *dh2, *dh1;
-    float *h1, *h2, *y3;
+    float4 *h1, *h2;  // pre-activations, quads of channels: [8][batch n^3]
+    float *y3;
     float *parts;
     int nparts;
     double *lparts, *loss;
@@ -915,8 +1055,26 @@ CnnPlan plan_for(int n, int batch)
     return pl;
 }
 
+// Planes of a run: the length that gives the CTA with most runs the fewest input
+// planes (each run reads two more than it writes).
+int conv_run(int n, int nb, int ctas)
+{
+    const long long cols = (long long)nb * ((n + TYT - 1) / TYT) * ((n + TXT - 1) / TXT);
+    int best = n;
+    long long best_t = 1LL << 60;
+    for (int chunks = 1; chunks <= n; ++chunks) {
+        const int run = (n + chunks - 1) / chunks;
+        const long long t = (cols * ((n + run - 1) / run) + ctas - 1) / ctas * (run + 2);
+        if (t < best_t) {
+            best_t = t;
+            best = run;
+        }
+    }
+    return best;
+}
+
 template <int CIN, int N, int EPI>
-cudaError_t conv(gbfd_cnn *c, const CUtensorMap &xmap, const ConvArgs &a)
+cudaError_t conv(gbfd_cnn *c, const CUtensorMap &xmap, ConvArgs a)
 {
     using SM = ConvSmem<CIN, N, EPI>;
     auto k = k_conv_tc<CIN, N, EPI>;
@@ -936,12 +1094,14 @@ cudaError_t conv(gbfd_cnn *c, const CUtensorMap &xmap, const ConvArgs &a)
             opted.fetch_or(bit);
     }
     const int n = a.n;
-    const long long ntiles = (long long)(a.npts / ((long long)n * n * n)) * ((n + ZB - 1) / ZB) *
-                             ((n + TYT - 1) / TYT) * ((n + TXT - 1) / TXT);
-    // persistent: one CTA per SM walking the tiles (fewer on request),
+    const int nb = (int)(a.npts / ((long long)n * n * n));
+    a.run = conv_run(n, nb, c->grid_conv);
+    const long long runs = (long long)nb * ((n + TYT - 1) / TYT) * ((n + TXT - 1) / TXT) *
+                           ((n + a.run - 1) / a.run);
+    // persistent: one CTA per SM walking the runs (fewer on request),
     // launched so that its prologue overlaps the previous kernel's tail
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<long long>(ntiles, c->grid_conv));
+    cfg.gridDim = dim3((unsigned)std::min<long long>(runs, c->grid_conv));
     cfg.blockDim = dim3(CONV_THREADS);
     cfg.dynamicSmemBytes = SM::BYTES;
     cfg.stream = c->stream;
@@ -971,8 +1131,8 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 
 // TMA map of a padded chunk-major activation of cin channels (B samples on
 // an n^3 grid): dims (8 (n + 2) values = x and the 8 channels of a chunk,
-// n + 2, (n + 2) B, cin / 8), box = one conv tile's halo, (8 HX, HY, HZ,
-// cin / 8): 160-byte rows.
+// n + 2, (n + 2) B, cin / 8), box = one haloed plane of a conv column, (8 HX, HY,
+// 1, cin / 8): 160-byte rows.
 bool encode_act_map(CUtensorMap *m, const bf16 *base, int n, int B, int cin)
 {
     PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
@@ -981,7 +1141,7 @@ bool encode_act_map(CUtensorMap *m, const bf16 *base, int n, int B, int cin)
     const cuuint64_t np2 = (cuuint64_t)(n + 2);
     const cuuint64_t dims[4] = {8 * np2, np2, np2 * (cuuint64_t)B, (cuuint64_t)(cin / 8)};
     const cuuint64_t strides[3] = {np2 * 16, np2 * np2 * 16, np2 * np2 * np2 * B * 16};
-    const cuuint32_t box[4] = {8 * HX, HY, HZ, (cuuint32_t)(cin / 8)};
+    const cuuint32_t box[4] = {8 * HX, HY, 1, (cuuint32_t)(cin / 8)};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(base), dims, strides, box,
               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -1106,7 +1266,7 @@ cudaError_t wgrad(gbfd_cnn *c, const CUtensorMap &amap, const CUtensorMap &bmap,
 cudaError_t backward(gbfd_cnn *c, const float *xs, const float *ts, int nf, int batch)
 {
     const int n3 = c->n * c->n * c->n, npts = batch * n3;
-    const int blocks = (npts + 255) / 256;
+    const int blocks = (npts + 256 * LOSS_PTS - 1) / (256 * LOSS_PTS);
     const float *sout = c->norm + 10;
     k_loss<<<blocks, 256, 0, c->stream>>>(c->y3, xs, ts, sout, nf, c->n, npts, c->batch,
                                           1.0f / ((float)NC * npts), c->dy3, c->lparts);
@@ -1215,8 +1375,8 @@ gbfd_status gbfd_cnn_init(int n, int batch, void *workspace, size_t workspace_by
     c->dy3 = (bf16 *)(b + pl.off[k++]);
     c->dh2 = (bf16 *)(b + pl.off[k++]);
     c->dh1 = (bf16 *)(b + pl.off[k++]);
-    c->h1 = (float *)(b + pl.off[k++]);
-    c->h2 = (float *)(b + pl.off[k++]);
+    c->h1 = (float4 *)(b + pl.off[k++]);
+    c->h2 = (float4 *)(b + pl.off[k++]);
     c->y3 = (float *)(b + pl.off[k++]);
     c->parts = (float *)(b + pl.off[k++]);
     c->lparts = (double *)(b + pl.off[k++]);

@@ -190,46 +190,49 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(MT, S::N) | tc::kIdescTransA | tc::kIdescTransB;
-            // MN-major, no swizzle: LBO = from 8 points to the next 8 (one row
-            // on), SBO = from one 8-channel chunk to the next
-            const uint64_t ad0 = tc::smem_desc(tc::smem_u32(smem), S::A_ROW, 128);
-            const uint64_t bd0 = tc::smem_desc(tc::smem_u32(smem + S::A_PITCH), S::B_ROW, S::B_CHUNK);
-            int i = 0;
-            for (; i < mine; ++i) {
-                const int s = i % NSTAGE, win = i / FLUSH, acc = win % NACC;
-                if (i % FLUSH == 0 &&
-                    !wait_or_abort(&acce[acc], ((win / NACC) & 1) ^ 1, abort))
-                    break;
-                if (!wait_or_abort(&full[s], (i / NSTAGE) & 1, abort))
-                    break;
-                cnt[1] = i + 1;
-                tc::fence_after_sync();
-                const uint64_t so = (uint64_t)((s * S::STAGE) >> 4);
-                const uint32_t d = tmem + acc * S::COLS;
-                const uint32_t keep = i % FLUSH != 0;
+        // the whole warp runs the loop, one lane issues (tc::mma_bf16_elect)
+        const uint32_t elected = tc::elect_one();
+        constexpr uint32_t idesc = tc::idesc_bf16_f32(MT, S::N) | tc::kIdescTransA | tc::kIdescTransB;
+        // MN-major, no swizzle: LBO = from 8 points to the next 8 (one row
+        // on), SBO = from one 8-channel chunk to the next
+        const uint64_t ad0 = tc::smem_desc(tc::smem_u32(smem), S::A_ROW, 128);
+        const uint64_t bd0 = tc::smem_desc(tc::smem_u32(smem + S::A_PITCH), S::B_ROW, S::B_CHUNK);
+        auto wait = [&](uint64_t *bar, int phase) {
+            return __all_sync(0xffffffffu, wait_or_abort(bar, phase, abort));
+        };
+        int i = 0;
+#pragma unroll 1
+        for (; i < mine; ++i) {
+            const int s = i % NSTAGE, win = i / FLUSH, acc = win % NACC;
+            if (i % FLUSH == 0 && !wait(&acce[acc], ((win / NACC) & 1) ^ 1))
+                break;
+            if (!wait(&full[s], (i / NSTAGE) & 1))
+                break;
+            cnt[1] = i + 1;
+            tc::fence_after_sync();
+            const uint64_t so = (uint64_t)((s * S::STAGE) >> 4);
+            const uint32_t d = tmem + acc * S::COLS;
+            const uint32_t keep = i % FLUSH != 0;
 #pragma unroll
-                for (int z = 0; z < ZB; ++z)
+            for (int z = 0; z < ZB; ++z)
 #pragma unroll
-                    for (int k = 0; k < KSTEPS; ++k)
+                for (int k = 0; k < KSTEPS; ++k)
 #pragma unroll
-                        for (int m = 0; m < S::NMMA; ++m)
-                            tc::mma_bf16(d + m * S::N,
-                                         ad0 + so + (uint64_t)((2 * k * S::A_ROW + z * 512) >> 4),
-                                         bd0 + so +
-                                             (uint64_t)((z * S::B_PLANE + 2 * k * S::B_ROW + m * 16) >> 4),
-                                         idesc, (z == 0 && k == 0) ? keep : 1u);
-                tc::commit(&empty[s]);
-                if (i % FLUSH == FLUSH - 1 || i == mine - 1) {
-                    tc::commit(&accf[acc]);
-                    cnt[2] = win + 1;
-                }
+                    for (int m = 0; m < S::NMMA; ++m)
+                        tc::mma_bf16_elect(
+                            elected, d + m * S::N,
+                            ad0 + so + (uint64_t)((2 * k * S::A_ROW + z * 512) >> 4),
+                            bd0 + so + (uint64_t)((z * S::B_PLANE + 2 * k * S::B_ROW + m * 16) >> 4),
+                            idesc, (z == 0 && k == 0) ? keep : 1u);
+            tc::commit_elect(elected, &empty[s]);
+            if (i % FLUSH == FLUSH - 1 || i == mine - 1) {
+                tc::commit_elect(elected, &accf[acc]);
+                cnt[2] = win + 1;
             }
-            if (i < mine) {  // a wait gave up: the MMAs issued so far are waited for below
-                tc::commit(stopped);
-                cnt[4] = 1;
-            }
+        }
+        if (i < mine) {  // a wait gave up: the MMAs issued so far are waited for below
+            tc::commit_elect(elected, stopped);
+            cnt[4] = 1;
         }
     } else if (warp == 3 || warp == 7) {
         // bias gradient: 8 channels of one point per 16-byte load; 8 lanes
