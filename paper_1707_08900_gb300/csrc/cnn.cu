@@ -202,7 +202,9 @@ constexpr int TAPS_XY = 9;  // (dy, dx) taps; dz is stacked along N
 // the first four warps of a group take the first half of the output channels.
 constexpr int EPI_WARPS = 8, EPI_GROUPS = 2;
 constexpr int CONV_THREADS = 32 * (2 + EPI_WARPS * EPI_GROUPS);
-constexpr int RING = 16;  // accumulator slots (output planes)
+constexpr int RING = 16;     // accumulator slots (output planes)
+constexpr int ACC_STEP = 4;  // slots that the MMAs claim at a time
+static_assert(RING % ACC_STEP == 0 && RING >= ACC_STEP + 3, "claimed slots were drained");
 
 template <int CIN, int NO, int EPI>
 struct ConvSmem {
@@ -367,7 +369,9 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(tslot);
+    // (the shuffle tells the compiler that the address is the warp's)
+    const uint32_t tmem =
+        __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(tslot), 0);
     // every MMA accumulates: the accumulators start at zero
     if (warp >= 2) {
         const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + c0;
@@ -443,31 +447,37 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             else
                 issue(ad, slot, dz0, std::integral_constant<int, 1>{});
         };
-        int i = 0, done = 0;  // planes loaded, output planes of earlier runs
+        // Between two planes' MMAs lies what the tensor pipe waits for, so it is
+        // kept short: counters instead of divisions, and the accumulator slots
+        // waited for and fenced ACC_STEP at a time.
+        int i = 0, s = 0, ph = 0;  // input planes so far; their stage and phase
+        int done = 0, o_next = 0;  // output planes of earlier runs; slots waited for
         bool ok = true;
         auto wait = [&](uint64_t *bar, int phase) {
-            ok = __all_sync(0xffffffffu, wait_or_abort(bar, phase, abort));
+            if (!tiled::mbar_try_wait(bar, phase))
+                ok = wait_or_abort(bar, phase, abort);
+            ok = __all_sync(0xffffffffu, ok);
             return ok;
         };
         each_run(n, nb, a.run, [&](int, int, int, int, int m) {
 #pragma unroll 1
-            for (int j = 0; j < m + 2; ++j, ++i) {
-                const int s = i % NSTAGE;
-                if (!wait(&full[s], (i / NSTAGE) & 1))
-                    return false;
-                cnt[1] = i + 1;
-                if (j < m) {  // output plane j begins: its slot must be drained and zero
-                    const int o = done + j;
-                    if (!wait(&acce[o % RING], ((o / RING) & 1) ^ 1))
-                        return false;
-                }
-                tc::fence_after_sync();
-                const uint64_t ad = ad0 + (uint64_t)((s * SM::A_PITCH) >> 4);
+            for (int j = 0; j < m + 2; ++j) {
                 // z taps whose output plane j - dz lies in the run, cut
                 // where the slots wrap
                 const int lo = max(0, j - m + 1), hi = min(2, j);
                 const int slot = (done + j - lo) % RING;
                 const int first = min(hi - lo + 1, slot + 1);
+                const uint64_t ad = ad0 + (uint64_t)((s * SM::A_PITCH) >> 4);
+                if (j < m && done + j == o_next) {
+                    // the next output planes: their slots must be drained and zero
+                    for (int k = 0; k < ACC_STEP; ++k, ++o_next)
+                        if (!wait(&acce[o_next % RING], ((o_next / RING) & 1) ^ 1))
+                            return false;
+                    tc::fence_after_sync();
+                }
+                if (!wait(&full[s], ph))
+                    return false;
+                cnt[1] = ++i;
                 issue_n(ad, slot, lo, first);
                 if (first < hi - lo + 1)
                     issue_n(ad, RING - 1, lo + first, hi - lo + 1 - first);
@@ -475,6 +485,10 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                 if (j >= 2) {
                     tc::commit_elect(elected, &accf[(done + j - 2) % RING]);
                     cnt[2] = done + j - 1;
+                }
+                if (++s == NSTAGE) {
+                    s = 0;
+                    ph ^= 1;
                 }
             }
             done += m;
