@@ -28,7 +28,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -679,7 +678,10 @@ __global__ void k_input_compact(const float *__restrict__ xs, int nf, int n, int
                                 const float *__restrict__ mean, const float *__restrict__ stdv,
                                 bf16 *__restrict__ x0)
 {
-    chain_next();  // the first convolution may start its prologue
+    // only then may the first convolution start its prologue, which reads the
+    // weights that the kernel before this one may have written
+    chain_wait();
+    chain_next();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= npts)
         return;
@@ -693,11 +695,12 @@ __global__ void k_input_compact(const float *__restrict__ xs, int nf, int n, int
 }
 
 // Same from a solver context's padded FP32 state (one box, batch 1).
-__global__ void k_input_state(const float *__restrict__ st, Layout L, int nf, int B,
+__global__ void k_input_state(const float *st, Layout L, int nf, int B,
                               const float *__restrict__ mean, const float *__restrict__ stdv,
                               bf16 *__restrict__ x0)
 {
-    chain_next();  // the first convolution may start its prologue
+    chain_wait();
+    chain_next();  // (after the wait, as above)
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = L.nx;
     if (p >= n * n * n)
@@ -711,19 +714,25 @@ __global__ void k_input_state(const float *__restrict__ st, Layout L, int nf, in
 }
 
 // state += std_out * y (the de-normalised predicted residual), ghosts kept.
-__global__ void k_apply(float *__restrict__ st, Layout L, int nf, const float *__restrict__ y,
-                        const float *__restrict__ sout)
+__global__ void k_apply(float *st, Layout L, int nf, const float *y, const float *sout)
 {
-    chain_wait();  // launched to overlap the last convolution's tail
+    chain_wait();
+    chain_next();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = L.nx;
     if (p >= n * n * n)
         return;
     const int z = p / (n * n), yy = (p / n) % n, x = p % n;
-    for (int f = 0; f < nf; ++f) {
-        const float v = st[lidx(L, f, z, yy, x)] + sout[f] * y[(long long)p * 8 + f];
-        store_ghosted(st, L, f, z, yy, x, v);
-    }
+    const float4 y4 = *reinterpret_cast<const float4 *>(y + (long long)p * 8);
+    const float yv[NC] = {y4.x, y4.y, y4.z, y4.w, y[(long long)p * 8 + 4]};
+    float v[NC];  // every load before the first store
+#pragma unroll
+    for (int f = 0; f < NC; ++f)
+        v[f] = f < nf ? st[lidx(L, f, z, yy, x)] + sout[f] * yv[f] : 0.f;
+#pragma unroll
+    for (int f = 0; f < NC; ++f)
+        if (f < nf)
+            store_ghosted(st, L, f, z, yy, x, v[f]);
 }
 
 // Normalised output [batch][5][n^3] from the layer-3 rows (tests, inference).
@@ -745,12 +754,14 @@ __global__ void k_output_compact(const float *__restrict__ y, int n3, int npts,
 // per thread: converting and adding every square in FP64 kept the narrow FP64
 // pipe busy for half of the kernel.
 constexpr int LOSS_PTS = 4;
-__global__ void __launch_bounds__(256) k_loss(const float *__restrict__ y, const float *__restrict__ xs,
+__global__ void __launch_bounds__(256) k_loss(const float *y, const float *__restrict__ xs,
                                               const float *__restrict__ ts,
                                               const float *__restrict__ sout, int nf, int n, int npts,
                                               int B, float inv_count, bf16 *__restrict__ dy3,
                                               double *__restrict__ part)
 {
+    chain_wait();
+    chain_next();
     const int n3 = n * n * n;
     __shared__ double sh[256];
     float hi = 0.f, lo = 0.f;
@@ -760,8 +771,8 @@ __global__ void __launch_bounds__(256) k_loss(const float *__restrict__ y, const
         if (p >= npts)
             break;
         const int b = p / n3, r = p - b * n3;
-        const float4 y4 = __ldg(reinterpret_cast<const float4 *>(y + (long long)p * 8));
-        const float yv[NC] = {y4.x, y4.y, y4.z, y4.w, __ldg(y + (long long)p * 8 + 4)};
+        const float4 y4 = *reinterpret_cast<const float4 *>(y + (long long)p * 8);
+        const float yv[NC] = {y4.x, y4.y, y4.z, y4.w, y[(long long)p * 8 + 4]};
         float d[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c)
@@ -793,8 +804,10 @@ __global__ void __launch_bounds__(256) k_loss(const float *__restrict__ y, const
         part[blockIdx.x] = sh[0];
 }
 
-__global__ void k_sum_double(const double *__restrict__ part, int n, double *__restrict__ out)
+__global__ void k_sum_double(const double *part, int n, double *__restrict__ out)
 {
+    chain_wait();
+    chain_next();
     __shared__ double sh[256];
     double s = 0.0;
     for (int i = threadIdx.x; i < n; i += 256)
@@ -825,6 +838,7 @@ struct PackArgs {
 // (dz', t') of 26 - tap (channels transposed).
 __global__ void k_adam_pack(PackArgs a)
 {
+    chain_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kParams)
         return;
@@ -1091,22 +1105,6 @@ template <int CIN, int N, int EPI>
 cudaError_t conv(gbfd_cnn *c, const CUtensorMap &xmap, ConvArgs a)
 {
     using SM = ConvSmem<CIN, N, EPI>;
-    auto k = k_conv_tc<CIN, N, EPI>;
-    // the shared-memory opt-in once per device (it is a per-device attribute
-    // of the kernel; the call costs host time on every launch otherwise)
-    static std::atomic<unsigned long long> opted{0};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess)
-        return e;
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (dev >= 64 || !(opted.load() & bit)) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SM::BYTES);
-        if (e != cudaSuccess)
-            return e;
-        if (dev < 64)
-            opted.fetch_or(bit);
-    }
     const int n = a.n;
     const int nb = (int)(a.npts / ((long long)n * n * n));
     a.run = conv_run(n, nb, c->grid_conv);
@@ -1114,19 +1112,10 @@ cudaError_t conv(gbfd_cnn *c, const CUtensorMap &xmap, ConvArgs a)
                            ((n + a.run - 1) / a.run);
     // persistent: one CTA per SM walking the runs (fewer on request),
     // launched so that its prologue overlaps the previous kernel's tail
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<long long>(runs, c->grid_conv));
-    cfg.blockDim = dim3(CONV_THREADS);
-    cfg.dynamicSmemBytes = SM::BYTES;
-    cfg.stream = c->stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, k, xmap, a);
     c->launches++;
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return launch_chained<k_conv_tc<CIN, N, EPI>>(
+        dim3((unsigned)std::min<long long>(runs, c->grid_conv)), dim3(CONV_THREADS), SM::BYTES, false,
+        c->stream, xmap, a);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
@@ -1209,9 +1198,15 @@ cudaError_t pack(gbfd_cnn *c, const float *g, float lr)
         a.bwd[l] = c->bwd[l];
         a.bias[l] = c->bias[l];
     }
-    k_adam_pack<<<(kParams + 255) / 256, 256, 0, c->stream>>>(a);
     c->launches++;
-    return cudaGetLastError();
+    return launch_chained<k_adam_pack>(dim3((kParams + 255) / 256), dim3(256), 0, false, c->stream, a);
+}
+
+cudaError_t stage_input(gbfd_cnn *c, const float *xs, int nf, int npts)
+{
+    return launch_chained<k_input_compact>(dim3((npts + 255) / 256), dim3(256), 0, false, c->stream,
+                                           xs, nf, c->n, npts, c->batch, (const float *)c->norm,
+                                           (const float *)(c->norm + 5), c->x0);
 }
 
 // forward of `npts` points whose layer-1 input is already in x0; `keep`
@@ -1251,11 +1246,6 @@ cudaError_t forward(gbfd_cnn *c, int npts, bool keep)
 template <int CO, int CI, bool WIDE, bool SWAP>
 cudaError_t wgrad(gbfd_cnn *c, const CUtensorMap &amap, const CUtensorMap &bmap, int npts, float *g)
 {
-    auto k = wg::k_wgrad_tc<WIDE>;
-    constexpr int smem = wg::Smem<WIDE>::BYTES;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return e;
     const int n = c->n;
     wg::Args a;
     a.n = n;
@@ -1266,14 +1256,15 @@ cudaError_t wgrad(gbfd_cnn *c, const CUtensorMap &amap, const CUtensorMap &bmap,
     const long long ntiles = (long long)a.nb * ((n + wg::ZB - 1) / wg::ZB) *
                              ((n + wg::TY - 1) / wg::TY) * ((n + wg::TX - 1) / wg::TX);
     const int grid = (int)std::min<long long>(ntiles, c->nparts);
-    k<<<grid, wg::THREADS, smem, c->stream>>>(amap, bmap, a);
-    e = cudaGetLastError();
+    constexpr int smem = wg::Smem<WIDE>::BYTES;
+    cudaError_t e = launch_chained<wg::k_wgrad_tc<WIDE>>(dim3(grid), dim3(wg::THREADS), smem, false,
+                                                         c->stream, amap, bmap, a);
     if (e != cudaSuccess)
         return e;
-    wg::k_wgrad_reduce<CO, CI, WIDE, SWAP>
-        <<<(wg::part_floats<WIDE>() + 31) / 32, 256, 0, c->stream>>>(c->parts, grid, g);
     c->launches += 2;
-    return cudaGetLastError();
+    return launch_chained<wg::k_wgrad_reduce<CO, CI, WIDE, SWAP>>(
+        dim3((wg::part_floats<WIDE>() + 31) / 32), dim3(256), 0, false, c->stream,
+        (const float *)c->parts, grid, g);
 }
 
 // loss, backward and gradients for `batch` samples (x0 and y3 from forward)
@@ -1282,11 +1273,14 @@ cudaError_t backward(gbfd_cnn *c, const float *xs, const float *ts, int nf, int 
     const int n3 = c->n * c->n * c->n, npts = batch * n3;
     const int blocks = (npts + 256 * LOSS_PTS - 1) / (256 * LOSS_PTS);
     const float *sout = c->norm + 10;
-    k_loss<<<blocks, 256, 0, c->stream>>>(c->y3, xs, ts, sout, nf, c->n, npts, c->batch,
-                                          1.0f / ((float)NC * npts), c->dy3, c->lparts);
-    k_sum_double<<<1, 256, 0, c->stream>>>(c->lparts, blocks, c->loss);
     c->launches += 2;
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained<k_loss>(dim3(blocks), dim3(256), 0, false, c->stream,
+                                           (const float *)c->y3, xs, ts, sout, nf, c->n, npts,
+                                           c->batch, 1.0f / ((float)NC * npts), c->dy3, c->lparts);
+    if (e != cudaSuccess)
+        return e;
+    e = launch_chained<k_sum_double>(dim3(1), dim3(256), 0, false, c->stream,
+                                     (const double *)c->lparts, blocks, c->loss);
     if (e != cudaSuccess)
         return e;
     // layer 3: weight gradient, then input gradient through GELU'(h2)
@@ -1570,9 +1564,7 @@ gbfd_status gbfd_cnn_forward(gbfd_cnn *c, const float *xs, int nf, int batch, fl
         return GBFD_ERR_INVALID_ARG;
     }
     const int n3 = c->n * c->n * c->n, npts = batch * n3;
-    k_input_compact<<<(npts + 255) / 256, 256, 0, c->stream>>>(xs, nf, c->n, npts, c->batch,
-                                                                c->norm, c->norm + 5, c->x0);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = stage_input(c, xs, nf, npts);
     if (e == cudaSuccess)
         e = forward(c, npts, false);
     if (e == cudaSuccess) {
@@ -1594,10 +1586,8 @@ gbfd_status gbfd_cnn_gradients(gbfd_cnn *c, const float *xs, const float *ts, in
         return GBFD_ERR_INVALID_ARG;
     }
     const int n3 = c->n * c->n * c->n, npts = batch * n3;
-    k_input_compact<<<(npts + 255) / 256, 256, 0, c->stream>>>(xs, nf, c->n, npts, c->batch,
-                                                                c->norm, c->norm + 5, c->x0);
+    cudaError_t e = stage_input(c, xs, nf, npts);
     c->launches++;
-    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
         e = forward(c, npts, true);
     if (e == cudaSuccess)
@@ -1625,10 +1615,8 @@ gbfd_status gbfd_cnn_train_step(gbfd_cnn *c, const float *xs, const float *ts, i
         return GBFD_ERR_INVALID_ARG;
     }
     const int n3 = c->n * c->n * c->n, npts = batch * n3;
-    k_input_compact<<<(npts + 255) / 256, 256, 0, c->stream>>>(xs, nf, c->n, npts, c->batch,
-                                                                c->norm, c->norm + 5, c->x0);
+    cudaError_t e = stage_input(c, xs, nf, npts);
     c->launches++;
-    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
         e = forward(c, npts, true);
     if (e == cudaSuccess)
@@ -1666,26 +1654,15 @@ gbfd_status gbfd_cnn_apply(gbfd_cnn *c, gbfd_ctx *ctx)
     // run on the solver's stream so the correction is ordered with its steps
     const cudaStream_t saved = c->stream;
     c->stream = s;
-    k_input_state<<<(n3 + 255) / 256, 256, 0, s>>>(st, L, nf, c->batch, c->norm, c->norm + 5,
-                                                   c->x0);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained<k_input_state>(dim3((n3 + 255) / 256), dim3(256), 0, false, s,
+                                                  (const float *)st, L, nf, c->batch,
+                                                  (const float *)c->norm,
+                                                  (const float *)(c->norm + 5), c->x0);
     if (e == cudaSuccess)
         e = forward(c, n3, false);
-    if (e == cudaSuccess) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((n3 + 255) / 256);
-        cfg.blockDim = dim3(256);
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, k_apply, st, L, nf, (const float *)c->y3,
-                               (const float *)(c->norm + 10));
-        if (e == cudaSuccess)
-            e = cudaGetLastError();
-    }
+    if (e == cudaSuccess)
+        e = launch_chained<k_apply>(dim3((n3 + 255) / 256), dim3(256), 0, false, s, st, L, nf,
+                                    (const float *)c->y3, (const float *)(c->norm + 10));
     c->stream = saved;
     c->launches += 2;
     return e == cudaSuccess ? GBFD_OK : ccuda(c, e, "cnn apply");

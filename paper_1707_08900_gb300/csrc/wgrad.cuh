@@ -154,7 +154,10 @@ __global__ void __launch_bounds__(THREADS, 1)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(tslot);
+    const uint32_t tmem =
+        __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(tslot), 0);
+    chain_wait();
+    chain_next();
 
     const int n = a.n;
     const int tx_n = (n + TX - 1) / TX, ty_n = (n + TY - 1) / TY, tz_n = (n + ZB - 1) / ZB;
@@ -376,9 +379,11 @@ __global__ void __launch_bounds__(THREADS, 1)
 // channel of A: see the operand stacking above; SWAP (layer 3): A is X and B
 // is dY, else A is dY.  Padding channels of g are set to zero.
 template <int CO, int CI, bool WIDE, bool SWAP>
-__global__ void __launch_bounds__(256) k_wgrad_reduce(const float *__restrict__ part, int nparts,
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float *part, int nparts,
                                                       float *__restrict__ g)
 {
+    chain_wait();
+    chain_next();
     constexpr int PF = part_floats<WIDE>();
     __shared__ float sh[8][32];
     const int lane = threadIdx.x % 32, grp = threadIdx.x / 32;
