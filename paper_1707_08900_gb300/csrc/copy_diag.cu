@@ -389,64 +389,82 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_diag_final(const double *__res
 // max |u|^2 alone, for the time-step rule: the same FP64 value as the full
 // reduction's, NaNs skipped as by fmax.  The FP64 pipe (2 lanes per SM and
 // clock) is what the full reduction waits for (its sums and exp(lnrho): 365 us
-// at 200 x 136 x 105), so FP32 storage looks at |u|^2 in FP32 first, whose
-// relative error is below 2^-22, and only values within 2^-20 of the largest
-// seen by the warp, or not comparable (overflow, NaN, tiny), are squared in
-// FP64.  A thread reads 16 bytes of each velocity component; the padded planes
-// are scanned as they lie (ghost columns and rows hold copies, padding zeros).
-// DRAM-bound: 11 us there.
+// at 200 x 136 x 105), so FP32 storage forms |u|^2 in FP32 first, whose relative
+// error is below 2^-22, and only values within 2^-20 of the block's largest, or
+// not comparable (overflow, NaN, tiny), are squared in FP64: about one per block
+// of 4096 points.
+// A thread reads UMAX_VEC times 16 bytes of each velocity component, all issued
+// before the first is used; the padded planes are scanned as they lie (ghost
+// columns and rows hold copies, padding zeros).
+constexpr int UMAX_VEC = 4;
 template <class TS>
 __global__ void __launch_bounds__(DIAG_THREADS) k_umax(const TS *__restrict__ st,
                                                        long long fpitch, long long nvec,
                                                        unsigned long long *__restrict__ out)
 {
     constexpr int V = 16 / sizeof(TS);
-    double best = 0.0;
-    float lim = 0.f;
-    for (long long base = (long long)blockIdx.x * DIAG_THREADS; base < nvec;
-         base += (long long)gridDim.x * DIAG_THREADS) {
-        const long long i = base + threadIdx.x;
-        uint4 q[3];
+    const long long base = (long long)blockIdx.x * (DIAG_THREADS * UMAX_VEC) + threadIdx.x;
+    uint4 q[UMAX_VEC][3];
+#pragma unroll
+    for (int k = 0; k < UMAX_VEC; ++k) {
+        const long long i = base + k * DIAG_THREADS;
 #pragma unroll
         for (int f = 0; f < 3; ++f)
-            q[f] = i < nvec ? __ldg(reinterpret_cast<const uint4 *>(st + (1 + f) * fpitch) + i)
-                            : make_uint4(0, 0, 0, 0);
-        const TS *a = reinterpret_cast<const TS *>(&q[0]), *b = reinterpret_cast<const TS *>(&q[1]),
-                 *c = reinterpret_cast<const TS *>(&q[2]);
-        auto exact = [&](int j) {
-            const double x = (double)a[j], y = (double)b[j], z = (double)c[j];
-            best = fmax(best, x * x + y * y + z * z);
-        };
-        if constexpr (sizeof(TS) == 8) {
+            q[k][f] = i < nvec ? __ldg(reinterpret_cast<const uint4 *>(st + (1 + f) * fpitch) + i)
+                               : make_uint4(0, 0, 0, 0);
+    }
+    double best = 0.0;
+    auto val = [&](int k, int f, int j) { return reinterpret_cast<const TS *>(&q[k][f])[j]; };
+    if constexpr (sizeof(TS) == 8) {
 #pragma unroll
-            for (int j = 0; j < V; ++j)
-                exact(j);
-        } else {
-            float s[V];
-            bool some = false;
+        for (int k = 0; k < UMAX_VEC; ++k)
 #pragma unroll
             for (int j = 0; j < V; ++j) {
-                s[j] = a[j] * a[j] + b[j] * b[j] + c[j] * c[j];
-                some = some || !(s[j] < lim);
+                const double x = val(k, 0, j), y = val(k, 1, j), z = val(k, 2, j);
+                best = fmax(best, x * x + y * y + z * z);
             }
-            if (__any_sync(0xffffffffu, some)) {
-                // the warp's largest comparable value first, then what comes
-                // within the FP32 error of it
-                float m = 0.f;
+    } else {
+        float s[UMAX_VEC][V], m = 0.f;
 #pragma unroll
-                for (int j = 0; j < V; ++j)
-                    m = s[j] < INFINITY ? fmaxf(m, s[j]) : m;
-                m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
-                if (m > 1e-30f)
-                    lim = fmaxf(lim, m * (1.f - 0x1p-20f));
+        for (int k = 0; k < UMAX_VEC; ++k)
 #pragma unroll
-                for (int j = 0; j < V; ++j)
-                    if (!(s[j] < lim))
-                        exact(j);
+            for (int j = 0; j < V; ++j) {
+                const float x = val(k, 0, j), y = val(k, 1, j), z = val(k, 2, j);
+                s[k][j] = x * x + y * y + z * z;
+                m = s[k][j] < INFINITY ? fmaxf(m, s[k][j]) : m;
             }
+        // (non-negative FP32 values order as their bits)
+        __shared__ unsigned sh[DIAG_THREADS / 32];
+        const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+        if (threadIdx.x % 32 == 0)
+            sh[threadIdx.x / 32] = wm;
+        __syncthreads();
+        unsigned bm = 0;
+#pragma unroll
+        for (int k = 0; k < DIAG_THREADS / 32; ++k)
+            bm = max(bm, sh[k]);
+        const float top = __uint_as_float(bm);
+        const float lim = top > 1e-30f ? top * (1.f - 0x1p-20f) : 0.f;
+        // a loop over the few, read again: unrolled and predicated, their FP64
+        // instructions take their slots in every warp (50 us instead of 5 at
+        // 200 x 136 x 105)
+        unsigned pick = 0;
+#pragma unroll
+        for (int k = 0; k < UMAX_VEC; ++k)
+#pragma unroll
+            for (int j = 0; j < V; ++j)
+                pick |= !(s[k][j] < lim) ? 1u << (k * V + j) : 0u;
+#pragma unroll 1
+        for (; pick; pick &= pick - 1) {
+            const int e = __ffs(pick) - 1;
+            const long long i = (base + e / V * DIAG_THREADS) * V + e % V;
+            const bool in = i < nvec * V;
+            const double x = in ? (double)st[fpitch + i] : 0.0, y = in ? (double)st[2 * fpitch + i] : 0.0,
+                         z = in ? (double)st[3 * fpitch + i] : 0.0;
+            best = fmax(best, x * x + y * y + z * z);
         }
     }
-    // (non-negative FP64 values order as their bits)
+    // (and non-negative FP64 values as theirs)
     unsigned long long v = (unsigned long long)__double_as_longlong(best);
     for (int k = 16; k > 0; k >>= 1)
         v = max(v, __shfl_xor_sync(0xffffffffu, v, k));
@@ -464,7 +482,7 @@ cudaError_t launch_umax(const void *state, const Layout &L, double *out, cudaStr
         return e;
     // whole planes: a multiple of 128 bytes, from a 16-byte aligned start
     const long long nvec = (long long)L.nz * L.plane * L.w / 16;
-    const int blocks = (int)std::min<long long>((nvec + DIAG_THREADS - 1) / DIAG_THREADS, 1216);
+    const unsigned blocks = (unsigned)((nvec + DIAG_THREADS * UMAX_VEC - 1) / (DIAG_THREADS * UMAX_VEC));
     if (L.w == 8)
         k_umax<double><<<blocks, DIAG_THREADS, 0, stream>>>((const double *)state, L.fpitch, nvec,
                                                            (unsigned long long *)out);
