@@ -522,6 +522,7 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
                 for (int a = 0; a < 3; ++a)
                     r[1 + a] = P::fma(P::bc(fo->amp32[a]), fc, r[1 + a]);
             }
+            unsigned redo = 0;  // results (field f, point p: bit 2 f + p) to form in FP64
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
                 const V u0 = colv[f][S];
@@ -538,24 +539,12 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
                     // the precision forms' update in float-float arithmetic;
                     // fexact: where that might round differently, in FP64
                     static_assert(std::is_same<TW, float>::value, "u-tilde stored in FP32");
+                    constexpr bool CHK = std::is_same<TA, fexact>::value;
                     V wn = first ? P::bc(0.f) : wv[f];
-                    const V wold = wn;
                     bool safe0 = true, safe1 = true;
-                    if constexpr (std::is_same<TA, fexact>::value) {
-                        rk3_pair_ff<true>(first, ffc, r[f], u0, wn, o2, safe0, safe1);
-                        if (!safe0) {
-                            wn.x = wold.x;
-                            rk3_update_f64<true, float>(first, alpha.d, beta.d, dt.d, r[f].x, u0.x,
-                                                        wn.x, o2.x);
-                        }
-                        if (!safe1) {
-                            wn.y = wold.y;
-                            rk3_update_f64<true, float>(first, alpha.d, beta.d, dt.d, r[f].y, u0.y,
-                                                        wn.y, o2.y);
-                        }
-                    } else {
-                        rk3_pair_ff<false>(first, ffc, r[f], u0, wn, o2, safe0, safe1);
-                    }
+                    rk3_pair_ff<CHK>(first, ffc, r[f], u0, wn, o2, safe0, safe1);
+                    if (CHK)
+                        redo |= (safe0 ? 0u : 1u << (2 * f)) | (safe1 ? 0u : 2u << (2 * f));
                     if (!last)
                         *reinterpret_cast<V *>(w + f * Lw.fpitch + go_w) = wn;
                 } else {
@@ -580,6 +569,37 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
                     *reinterpret_cast<V *>(op + gdy) = o2;
                     if (gdx)
                         *reinterpret_cast<V *>(op + gdy + gdx) = o2;
+                }
+            }
+            if constexpr (std::is_same<TA, fexact>::value) {
+                // out of the way of the rest: one copy of the code, values
+                // picked by selects, the results stored over the others
+                while (redo) {
+                    const int bit = __ffs(redo) - 1, f = bit >> 1, pt = bit & 1;
+                    redo &= redo - 1;
+                    V rf = r[0], uf = colv[0][S];
+#pragma unroll
+                    for (int k = 1; k < NF; ++k) {
+                        rf = f == k ? r[k] : rf;
+                        uf = f == k ? colv[k][S] : uf;
+                    }
+                    float wn = 0.f, on;
+                    if (need_w)
+                        wn = *(reinterpret_cast<const TW *>(wsm + ((wrun + o) % NW) * RG::WSLOT_PITCH) +
+                               f * TX * TY + ty * TX + 2 * tx + pt);
+                    rk3_update_f64<true, float>(first, alpha.d, beta.d, dt.d, pt ? rf.y : rf.x,
+                                                pt ? uf.y : uf.x, wn, on);
+                    if (!last)
+                        w[f * Lw.fpitch + go_w + pt] = wn;
+                    float *op = out + f * Ls.fpitch + go_s + pt;
+                    *op = on;
+                    if (gdx)
+                        op[gdx] = on;
+                    if (gdy) {
+                        op[gdy] = on;
+                        if (gdx)
+                            op[gdy + gdx] = on;
+                    }
                 }
             }
         }

@@ -18,7 +18,7 @@ cudaError_t launch_substep_tiled(const StateBufs &b, const Coef<TS> &c, const RK
     // its update in float-float arithmetic with the few results that could
     // round differently redone in FP64 (the same bits as the FP64 update of the
     // same right-hand side, without its 15 FP64 operations per point on a pipe
-    // of 2 lanes per SM and clock): 1179 -> 475 us per substep at 256^3
+    // of 2 lanes per SM and clock): 1179 -> 384 us per substep at 256^3
     if constexpr (sizeof(TW) == 4)
         if (cfg < 0 && form == 0)
             return launch_lag_exact(b, c, st, nf, b.zc, dev_error, cache, stream, launches);
