@@ -164,22 +164,23 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
     // local state plane j is grid plane z0 - 3 + j (wrapped), copy jrun + j
     // of this CTA: slot (jrun + j) % NS, phase ((jrun + j) / NS) & 1
     int issued = 0, wissued = 0;
+    const bool copier = threadIdx.x < 32;  // the warp that issues the copies
+    const uint32_t elected = tiled::elect_one();
     auto issue = [&](int j) {
         if (j == skip_plane)  // fault injection for the bounded-wait test
             return;
         int z = z0 - R + j;
         z = zplane(Ls, z) + Ls.gz;  // TMA z coordinate
-        const int slot = (jrun + j) % NS;
-        tiled::mbar_expect_tx(&bars[slot], RG::SLOT_BYTES);
-        tiled::tma_load_4d(smem + slot * RG::SLOT_PITCH, tmap, &bars[slot], x0, y0, z, 0);
+        const int slot = (unsigned)(jrun + j) % NS;
+        tiled::tma_load_4d_elect(elected, smem + slot * RG::SLOT_PITCH, tmap, &bars[slot],
+                                 RG::SLOT_BYTES, x0, y0, z, 0);
     };
     auto issue_w = [&](int o) {
-        const int slot = (wrun + o) % NW;
-        tiled::mbar_expect_tx(&wbars[slot], RG::WSLOT_BYTES);
-        tiled::tma_load_4d(wsm + slot * RG::WSLOT_PITCH, wmap, &wbars[slot], x0 + GX, y0 + GY,
-                           z0 + o, 0);
+        const int slot = (unsigned)(wrun + o) % NW;
+        tiled::tma_load_4d_elect(elected, wsm + slot * RG::WSLOT_PITCH, wmap, &wbars[slot],
+                                 RG::WSLOT_BYTES, x0 + GX, y0 + GY, z0 + o, 0);
     };
-    if (threadIdx.x == 0) {
+    if (copier) {
         tiled::fence_proxy_async();
 #pragma unroll 1
         for (int j = 0; j < NS && j < nplanes; ++j)
@@ -666,7 +667,7 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
     auto top = [&](const int s0) -> bool {
         if (__syncthreads_or(timeout))
             return true;
-        if (threadIdx.x == 0) {
+        if (copier) {
             tiled::fence_proxy_async();
             const int jend = min(s0 + NS, nplanes);
 #pragma unroll 1

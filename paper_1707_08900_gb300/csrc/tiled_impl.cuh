@@ -101,6 +101,30 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, u
         : "memory");
 }
 
+// One lane of the (converged) warp, and the copy that it issues when the whole
+// warp reaches the code: the loop around stays uniform, without the divergence
+// and the per-thread arithmetic of a branch for one thread.
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(p));
+    return p;
+}
+__device__ __forceinline__ void tma_load_4d_elect(uint32_t elected, void *dst, const CUtensorMap *map,
+                                                  uint64_t *bar, uint32_t bytes, int c0, int c1,
+                                                  int c2, int c3)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %8, 0;\n\t"
+        "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%2], %7;\n\t"
+        "@q cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2];\n\t}" ::"r"(smem_u32(dst)),
+        "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bytes),
+        "r"(elected)
+        : "memory");
+}
+
 // Accessor over the plane ring: dz selects the plane, (dy, dx) the offset in
 // it; the thread's own z-column comes from the sliding register window.
 template <class TS, int NF, int BX, int FSTRIDE>
