@@ -167,22 +167,23 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
     // local state plane j is grid plane z0 - 3 + j (wrapped); it is copy
     // jrun + j of this CTA: slot (jrun + j) % NS, phase (jrun + j) / NS
     int issued = 0, wissued = 0;
+    const bool copier = threadIdx.x < 32;  // the warp that issues the copies
+    const uint32_t elected = tiled::elect_one();
     auto issue = [&](int j) {
         // fault injection for the bounded-wait test: never copy this plane
         if (j == skip_plane)
             return;
         int z = z0 - R + j;
         z = zplane(Ls, z) + Ls.gz;  // TMA z coordinate
-        const int slot = (jrun + j) % NS;
-        tiled::mbar_expect_tx(&bars[slot], RG::SLOT_BYTES);
-        tiled::tma_load_4d(smem + slot * RG::SLOT_PITCH, tmap, &bars[slot], x0, y0, z, 0);
+        const int slot = (unsigned)(jrun + j) % NS;
+        tiled::tma_load_4d_elect(elected, smem + slot * RG::SLOT_PITCH, tmap, &bars[slot],
+                                 RG::SLOT_BYTES, x0, y0, z, 0);
     };
     auto issue_w = [&](int o) {
         if constexpr (!WG) {
-            const int slot = (wrun + o) % NW;
-            tiled::mbar_expect_tx(&wbars[slot], RG::WSLOT_BYTES);
-            tiled::tma_load_4d(wsm + slot * RG::WSLOT_PITCH, wmap, &wbars[slot], x0 + GX, y0 + GY,
-                               z0 + o, 0);
+            const int slot = (unsigned)(wrun + o) % NW;
+            tiled::tma_load_4d_elect(elected, wsm + slot * RG::WSLOT_PITCH, wmap, &wbars[slot],
+                                     RG::WSLOT_BYTES, x0 + GX, y0 + GY, z0 + o, 0);
         }
     };
     // The forward-accumulated and 19-point forms read only the centre plane
@@ -192,7 +193,7 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
     constexpr bool FWD = PK && MIXED;
     constexpr int LAG = (MIXED && !FWD) ? 0 : R;
     static_assert(NS >= 4 && NS >= (LAG ? U + 3 : U + 6), "ring too short for the planes in use");
-    if (threadIdx.x == 0) {
+    if (copier) {
         tiled::fence_proxy_async();
 #pragma unroll 1
         for (int j = 0; j < NS && j < nplanes; ++j)
@@ -276,7 +277,7 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
             // a ring shorter than the six leading planes: the first ones are
             // consumed, their slots take the rest
             __syncthreads();
-            if (threadIdx.x == 0) {
+            if (copier) {
                 tiled::fence_proxy_async();
 #pragma unroll 1
                 for (int jj = NS; jj < 2 * R; ++jj)
@@ -860,7 +861,7 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
         // any thread ends the CTA for everyone
         if (__syncthreads_or(timeout))
             break;
-        if (threadIdx.x == 0) {
+        if (copier) {
             tiled::fence_proxy_async();
             const int jend = min(o + LAG + NS, nplanes);
 #pragma unroll 1

@@ -143,13 +143,15 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
     const int skip_plane = blockIdx.x == 0 && blockIdx.y == 0 ? skip_plane_arg : -1;
 
     int issued = 0;
+    const bool copier = threadIdx.x < 32;  // the warp that issues the copies
+    const uint32_t elected = tiled::elect_one();
     auto issue = [&](int j) {
         if (j == skip_plane)  // fault injection for the bounded-wait test
             return;
         const int z = zplane(Ls, z0 - R + j) + Ls.gz;  // TMA z coordinate
         const int slot = j % NS;
-        tiled::mbar_expect_tx(&bars[slot], RG::SLOT_BYTES);
-        tiled::tma_load_4d(smem + slot * RG::SLOT_PITCH, &tmap, &bars[slot], x0, y0, z, 0);
+        tiled::tma_load_4d_elect(elected, smem + slot * RG::SLOT_PITCH, &tmap, &bars[slot],
+                                 RG::SLOT_BYTES, x0, y0, z, 0);
     };
     auto issue_upto = [&](int jend) {
         jend = min(jend, nplanes);
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
             timeout = true;
         waited = j + 1;
     };
-    if (threadIdx.x == 0) {
+    if (copier) {
         tiled::fence_proxy_async();
         issue_upto(NS);
     }
@@ -237,7 +239,7 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
     if (__syncthreads_or(timeout)) {
         timeout = true;
     } else {
-        if (threadIdx.x == 0) {
+        if (copier) {
             tiled::fence_proxy_async();
             issue_upto(R + NS);
         }
@@ -418,7 +420,7 @@ __global__ void __launch_bounds__(TX *TY, MINB) k_substep_lag64(
     auto top = [&](const int s) -> bool {
         if (__syncthreads_or(timeout))
             return true;
-        if (threadIdx.x == 0) {
+        if (copier) {
             tiled::fence_proxy_async();
             issue_upto(s + NS);
         }
