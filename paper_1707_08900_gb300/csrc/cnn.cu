@@ -940,7 +940,7 @@ __global__ void __launch_bounds__(256) k_box_filter_ff(const float *__restrict__
         s = t;
         e = __fadd_rn(e, d);
     };
-#pragma unroll 1
+#pragma unroll(RR <= 4 ? 2 * H + 1 : 1)
     for (int a = -H; a <= H; ++a) {
         int z = RR * Z + a;
         z = z < 0 ? z + L.nz : (z >= L.nz ? z - L.nz : z);
