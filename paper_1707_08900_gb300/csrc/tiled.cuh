@@ -84,6 +84,23 @@ cudaError_t launch_lag_shfl(const StateBufs &b, const Coef<float> &c, const RKSt
                             int zc, int cfg_key, int *dev_error, TmapCache *cache,
                             cudaStream_t stream, int *launches);
 
+// Whether a grid is large enough for kernels instantiated per RK3 substep.  They
+// drop run-time tests from the plane loop (about 7% of the FP32 kernel), but three
+// kernels taking turns find their code gone from the instruction caches, which
+// costs every launch 1 to 4 us.  Measured per substep, one kernel against three:
+// 32^3 4.2 and 5.1 us, 64^3 9.8 and 11.1, 96^3 19.2 and 21.5, 120 x 110 x 100
+// 35.3 and 39.7; 128^3 43.5 and 41.2, 200 x 136 x 105 52.6 and 48.6, 576 x 512 x
+// 452 8% in favour of three (160^3, one wave of CTAs, 71.1 and 74.7).
+inline bool stage_kernels(const Layout &L)
+{
+    return (long long)L.nx * L.ny * L.nz >= (1LL << 21);
+}
+
+// The default kernel's per-substep instantiations for grids that are not whole
+// tiles, four fields or unequal spacings (tiled_f32_stage.cu; unforced).
+cudaError_t launch_lag_stage(const StateBufs &b, const RKStage &st, int nf, int zc, int cfg_key,
+                             int *dev_error, TmapCache *cache, cudaStream_t stream, int *launches);
+
 // The FP64-update precision form (u-tilde in FP32, 55-point form) on the FP32
 // default kernel (tiled_ff.cu).
 cudaError_t launch_lag_exact(const StateBufs &b, const Coef<float> &c, const RKStage &st, int nf,

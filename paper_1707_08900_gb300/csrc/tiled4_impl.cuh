@@ -841,8 +841,8 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
         }                                                                                         \
         GBFD_LAUNCH_LAG_C(NFV, FRC, FoldCoef<float>, fc);                                              \
     } while (0)
-    // the five-field isotropic case on whole tiles (forced steps in FP32
-    // arithmetic included): the substep is a template argument and the
+    // the five-field isotropic case on whole tiles of a large grid (forced steps
+    // in FP32 arithmetic included): the substep is a template argument and the
     // grid-extent test goes
     constexpr bool SPEC = TM && MINB == 1 && !ICVT && !SHFL && std::is_same<TW, float>::value &&
                           (std::is_same<TA, float>::value || std::is_same<TA, ffloat>::value ||
@@ -852,7 +852,7 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
         // forced steps too, in FP32 arithmetic (the forcing is a compile-time
         // switch of the same kernel)
         const bool frc_ok = !st.fo.on || std::is_same<TA, float>::value;
-        if (nf == 5 && frc_ok && iso && full && st.s >= 0 && st.s <= 2) {
+        if (nf == 5 && frc_ok && iso && full && stage_kernels(b.Ls) && st.s >= 0 && st.s <= 2) {
 #define GBFD_LAUNCH_LAG_S(FRC, SV)                                                                \
     do {                                                                                          \
         constexpr auto kern = tiled4::k_substep_lag<TW, TA, 5, TX, TY, NS, U, MINB, ICVT, FRC,    \
