@@ -406,9 +406,9 @@ const char *gbfd_batch_last_error(const gbfd_batch *b);
  * net = conv3 . GELU . conv2 . GELU . conv1, each a periodic 3x3x3
  * cross-correlation y[o,p] = b[o] + sum_{c,t} W[o,c,t] x[c,p+t] (channels
  * 5 -> 32 -> 32 -> 5, exact GELU).  BF16 weights and activations, FP32
- * accumulation: the convolutions and their input gradients run as
- * implicit GEMMs on the tcgen05 tensor cores; weight gradients are FP32
- * sums over the grid; Adam keeps FP32 master weights.
+ * accumulation: the convolutions, their input gradients and the weight
+ * gradients (sums over the grid) run on the tcgen05 tensor cores; Adam keeps
+ * FP32 master weights.
  * Compact state arrays are [batch][5][n][n][n] FP32 on the device (the fifth
  * channel is ignored when nf = 4).  Parameters are exchanged in FP32, layer
  * by layer: W1 [32][5][3][3][3], b1 [32], W2 [32][32][3][3][3], b2 [32],

@@ -200,7 +200,6 @@ StateBufs bufs(gbfd_ctx *c)
     b.div = c->div_region ? c->div_region + c->Ld.origin : nullptr;
     b.Ls = c->Ls;
     b.Lw = c->Lw;
-    b.cd = &c->c64;
     b.zc = c->zc;
     return b;
 }

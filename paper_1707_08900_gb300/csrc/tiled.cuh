@@ -35,9 +35,9 @@ constexpr int kZcChoices = 5;
 //      per iteration
 //   3  the same with one step per iteration
 //   4  the same as 2 with the pending right-hand sides in TMEM (default;
-//      on whole tiles with equal spacing and five unforced fields it runs an
-//      instantiation per RK3 substep, the substep and the grid-extent test
-//      fixed at compile time)
+//      on large grids it runs an instantiation per RK3 substep, the substep
+//      and on whole tiles the grid-extent test fixed at compile time, see
+//      stage_kernels below)
 //   5  the same as 4 compiled for three CTAs per SM (168 registers; slower:
 //      13.3 against 19.2 G updates/s at 256^3, spills and still two CTAs per
 //      SM, whose shared memory the ring fills; kept as the check that its
@@ -52,9 +52,9 @@ constexpr int kDefaultF32 = kVarLagTm * kZcChoices;
 // Default FP64 table entry (see tiled_f64.cu): the one-point kernel with the
 // output lagged three planes behind the in-plane work (z-paired Eq. 8 terms
 // from each centre plane's own differences), 16 x 8 tiles, a 5-slot ring for
-// three CTAs per SM, z-chunks of 40: 0.622 against 0.554 G updates/s for the
-// one-point kernel that reads every stencil point (entry 5) at 256^3; the
-// FP64 pipe is the bound.
+// three CTAs per SM: 0.72 against 0.554 G updates/s for the one-point kernel
+// that reads every stencil point (entry 5) at 256^3 (0.622 before the weights
+// were folded); the FP64 pipe is the bound.
 constexpr int kDefaultF64 = 5 * kZcChoices;
 
 // Tile tables per storage width (4 = FP32 storage, 8 = FP64 storage).
@@ -98,8 +98,9 @@ inline bool stage_kernels(const Layout &L)
 
 // The default kernel's per-substep instantiations for grids that are not whole
 // tiles, four fields or unequal spacings (tiled_f32_stage.cu; unforced).
-cudaError_t launch_lag_stage(const StateBufs &b, const RKStage &st, int nf, int zc, int cfg_key,
-                             int *dev_error, TmapCache *cache, cudaStream_t stream, int *launches);
+cudaError_t launch_lag_stage(const StateBufs &b, const Coef<float> &c, const RKStage &st, int nf,
+                             int zc, int cfg_key, int *dev_error, TmapCache *cache,
+                             cudaStream_t stream, int *launches);
 
 // The FP64-update precision form (u-tilde in FP32, 55-point form) on the FP32
 // default kernel (tiled_ff.cu).

@@ -22,9 +22,12 @@
 // three halo planes below and above a z-chunk are never centres: their arm
 // differences come from loads of their own.
 //
-// The weights are folded (FoldCoef, common.cuh): viscosity, signs and, with the
-// FP32 update, the time step are in the stencil weights, so every derivative
-// goes straight into the right-hand side.
+// With folded weights (FoldCoef, common.cuh; the batch's lagged routine) every
+// derivative goes straight into the right-hand side: 3% faster at 256^3 (3.40 and
+// 3.30 ms for four steps).  The single box does not take them: all terms round
+// against the largest one, VC u, which grows with nu dt / h^2, and at 512^3 two
+// steps are 7.5e-8 from the 64-bit result instead of 6.0e-8; the batch's boxes are
+// small (VC below 0.4) and as near with either (6.7e-8).
 //
 // Per output plane and thread this reads 92 shared pairs (5 column values,
 // 50 x/y arms of the five fields, 32 for the two (x, y) cross terms, 5 of
@@ -130,6 +133,7 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
     constexpr int NW = RG::NW;
     constexpr int NTX = TX / 2;
     constexpr bool UP32 = std::is_same<TA, float>::value && std::is_same<TW, float>::value;
+    constexpr bool FOLD = is_fold<CoefT>::value;
     // the prologue holds local planes 0..5 at once; each step reads its
     // centre plane and the plane three above it
     static_assert(NS >= 6 && NS >= U + 4, "ring too short");
@@ -225,12 +229,16 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
 
     const V NEG1 = P::bc(-1.f);
     // add the arm differences d[k-1] of one plane, ac index MC, with weights
-    // M3(pair, k): plus to the outputs below it, minus to those above
+    // M3 or MX (pair, k): plus to the outputs below it, minus to those above
     auto spread = [&](V *ac, const V *d, int pair, auto mcc) {
         constexpr int MC = decltype(mcc)::value;
 #pragma unroll
         for (int k = 1; k <= 3; ++k) {
-            const float mk = c.M3(pair, k);
+            float mk;
+            if constexpr (FOLD)
+                mk = c.M3(pair, k);
+            else
+                mk = c.MX(pair, k);
             if (MC - k >= 0)
                 ac[MC - k] = P::fma(P::bc(mk), d[k - 1], ac[MC - k]);
             if (MC + k < W)
@@ -359,122 +367,260 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
         auto ld2 = [&](int f, int dy, int dx) -> V {
             return *reinterpret_cast<const V *>(sm + cb + f * FSTRIDE + dy * BX + dx);
         };
-        V g[3], h[3], gd[3], y1p, y1m;
-        // Eqs. 6-7 of field f: the gradient (LN: grad lnrho, else the folded
-        // -s grad) into g, the weighted second derivatives of velocity
-        // component I >= 0 onto acc; h, gd keep the x and y differences
-        auto axial = [&](int f, auto lc, auto ic, V &acc) {
-            constexpr bool LN = decltype(lc)::value;
-            constexpr int I = decltype(ic)::value;
-            auto w1 = [&](int a, int k) { return P::bc(LN ? c.L1(a, k) : c.N1(a, k)); };
-            auto w2 = [&](int a, int k) { return P::bc(a == I ? c.X2(a, k) : c.V2(a, k)); };
-            const V cc = C(f, 3);
-            V m4, m2, p2, p4;
-            xnb(cb + f * FSTRIDE, cc, m4, m2, p2, p4);
-            xdiff(m4, m2, cc, p2, p4, h);
-            g[0] = P::fma(w1(0, 3), h[2], P::fma(w1(0, 2), h[1], P::mul(w1(0, 1), h[0])));
-            if constexpr (I >= 0) {
-                const V s1 = P::mk(cc.y + m2.y, p2.x + cc.x);
-                const V s3 = P::mk(p2.y + m4.y, p4.x + m2.x);
-                acc = P::fma(w2(0, 3), s3,
-                             P::fma(w2(0, 2), P::add(p2, m2), P::fma(w2(0, 1), s1, acc)));
-            }
-            V byz;
-#pragma unroll
-            for (int k = 1; k <= 3; ++k) {
-                const V yp = ld2(f, k, 0), ym = ld2(f, -k, 0);
-                if (k == 1) {
-                    y1p = yp;
-                    y1m = ym;
-                }
-                const V zp = C(f, 3 + k), zm = C(f, 3 - k);
-                const V dyv = P::fma(ym, NEG1, yp), dzv = P::fma(zm, NEG1, zp);
-                gd[k - 1] = dyv;
-                g[1] = k == 1 ? P::mul(w1(1, 1), dyv) : P::fma(w1(1, k), dyv, g[1]);
-                g[2] = k == 1 ? P::mul(w1(2, 1), dzv) : P::fma(w1(2, k), dzv, g[2]);
+        if constexpr (FOLD) {
+            V g[3], h[3], gd[3], y1p, y1m;
+            // Eqs. 6-7 of field f: the gradient (LN: grad lnrho, else the folded
+            // -s grad) into g, the weighted second derivatives of velocity
+            // component I >= 0 onto acc; h, gd keep the x and y differences
+            auto axial = [&](int f, auto lc, auto ic, V &acc) {
+                constexpr bool LN = decltype(lc)::value;
+                constexpr int I = decltype(ic)::value;
+                auto w1 = [&](int a, int k) { return P::bc(LN ? c.L1(a, k) : c.N1(a, k)); };
+                auto w2 = [&](int a, int k) { return P::bc(a == I ? c.X2(a, k) : c.V2(a, k)); };
+                const V cc = C(f, 3);
+                V m4, m2, p2, p4;
+                xnb(cb + f * FSTRIDE, cc, m4, m2, p2, p4);
+                xdiff(m4, m2, cc, p2, p4, h);
+                g[0] = P::fma(w1(0, 3), h[2], P::fma(w1(0, 2), h[1], P::mul(w1(0, 1), h[0])));
                 if constexpr (I >= 0) {
-                    byz = k == 1 ? P::mul(w2(1, 1), P::add(yp, ym))
-                                 : P::fma(w2(1, k), P::add(yp, ym), byz);
-                    byz = P::fma(w2(2, k), P::add(zp, zm), byz);
+                    const V s1 = P::mk(cc.y + m2.y, p2.x + cc.x);
+                    const V s3 = P::mk(p2.y + m4.y, p4.x + m2.x);
+                    acc = P::fma(w2(0, 3), s3,
+                                 P::fma(w2(0, 2), P::add(p2, m2), P::fma(w2(0, 1), s1, acc)));
                 }
-            }
-            if constexpr (I >= 0)
-                acc = P::add(acc, byz);
-        };
-        // Eq. 8 in the (x, y) plane, onto acc: D_xy f = sum_k MX_k [h_k(y+k) -
-        // h_k(y-k)]; the centre pairs of rows y+-1 are those of the y arm just
-        // loaded
-        auto mix_xy = [&](int f, V &acc) {
+                V byz;
 #pragma unroll
-            for (int k = 1; k <= 3; ++k) {
-                V hh[2];
-#pragma unroll
-                for (int sgn = 0; sgn < 2; ++sgn) {
-                    const int dy = sgn ? -k : k;
-                    const V m2 = ld2(f, dy, -2), p2 = ld2(f, dy, 2);
+                for (int k = 1; k <= 3; ++k) {
+                    const V yp = ld2(f, k, 0), ym = ld2(f, -k, 0);
                     if (k == 1) {
-                        const V cc = sgn ? y1m : y1p;
-                        hh[sgn] = P::mk(cc.y - m2.y, p2.x - cc.x);
-                    } else if (k == 2) {
-                        hh[sgn] = P::fma(m2, NEG1, p2);
-                    } else {
-                        const V m4 = ld2(f, dy, -4), p4 = ld2(f, dy, 4);
-                        hh[sgn] = P::mk(p2.y - m4.y, p4.x - m2.x);
+                        y1p = yp;
+                        y1m = ym;
+                    }
+                    const V zp = C(f, 3 + k), zm = C(f, 3 - k);
+                    const V dyv = P::fma(ym, NEG1, yp), dzv = P::fma(zm, NEG1, zp);
+                    gd[k - 1] = dyv;
+                    g[1] = k == 1 ? P::mul(w1(1, 1), dyv) : P::fma(w1(1, k), dyv, g[1]);
+                    g[2] = k == 1 ? P::mul(w1(2, 1), dzv) : P::fma(w1(2, k), dzv, g[2]);
+                    if constexpr (I >= 0) {
+                        byz = k == 1 ? P::mul(w2(1, 1), P::add(yp, ym))
+                                     : P::fma(w2(1, k), P::add(yp, ym), byz);
+                        byz = P::fma(w2(2, k), P::add(zp, zm), byz);
                     }
                 }
-                acc = P::fma(P::bc(c.M3(0, k)), P::fma(hh[1], NEG1, hh[0]), acc);
+                if constexpr (I >= 0)
+                    acc = P::add(acc, byz);
+            };
+            // Eq. 8 in the (x, y) plane, onto acc: D_xy f = sum_k MX_k [h_k(y+k) -
+            // h_k(y-k)]; the centre pairs of rows y+-1 are those of the y arm just
+            // loaded
+            auto mix_xy = [&](int f, V &acc) {
+#pragma unroll
+                for (int k = 1; k <= 3; ++k) {
+                    V hh[2];
+#pragma unroll
+                    for (int sgn = 0; sgn < 2; ++sgn) {
+                        const int dy = sgn ? -k : k;
+                        const V m2 = ld2(f, dy, -2), p2 = ld2(f, dy, 2);
+                        if (k == 1) {
+                            const V cc = sgn ? y1m : y1p;
+                            hh[sgn] = P::mk(cc.y - m2.y, p2.x - cc.x);
+                        } else if (k == 2) {
+                            hh[sgn] = P::fma(m2, NEG1, p2);
+                        } else {
+                            const V m4 = ld2(f, dy, -4), p4 = ld2(f, dy, 4);
+                            hh[sgn] = P::mk(p2.y - m4.y, p4.x - m2.x);
+                        }
+                    }
+                    acc = P::fma(P::bc(c.M3(0, k)), P::fma(hh[1], NEG1, hh[0]), acc);
+                }
+            };
+            using NoComp = std::integral_constant<int, -1>;
+            const V uc[3] = {C(1, 3), C(2, 3), C(3, 3)};
+            const V NNU = P::bc(c.nnu);
+            V acc[3], gl[3], nng[3], q[3], dvm;
+            axial(0, std::true_type{}, NoComp{}, acc[0]);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                gl[a] = g[a];
+                nng[a] = P::mul(NNU, g[a]);
+                q[a] = P::fma(NNU, g[a], uc[a]);
             }
-        };
-        using NoComp = std::integral_constant<int, -1>;
-        const V uc[3] = {C(1, 3), C(2, 3), C(3, 3)};
-        const V NNU = P::bc(c.nnu);
-        V acc[3], gl[3], nng[3], q[3], dvm;
-        axial(0, std::true_type{}, NoComp{}, acc[0]);
+            auto component = [&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                acc[i] = i == 0 ? P::mul(P::bc(c.VC(0)), uc[0])
+                                : P::fma(P::bc(c.VC(i)), uc[i], acc[i]);
+                axial(1 + i, std::false_type{}, ic, acc[i]);
+                // the arm differences of this plane, in the same order as a halo plane's
+                if constexpr (i == 0) {
+                    spread(acz, h, 1, std::integral_constant<int, MC>{});
+                } else if constexpr (i == 1) {
+                    spread(acz, gd, 2, std::integral_constant<int, MC>{});
+                } else {
+                    spread(acx, h, 1, std::integral_constant<int, MC>{});
+                    spread(acy, gd, 2, std::integral_constant<int, MC>{});
+                }
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            gl[a] = g[a];
-            nng[a] = P::mul(NNU, g[a]);
-            q[a] = P::fma(NNU, g[a], uc[a]);
-        }
-        auto component = [&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            acc[i] = i == 0 ? P::mul(P::bc(c.VC(0)), uc[0])
-                            : P::fma(P::bc(c.VC(i)), uc[i], acc[i]);
-            axial(1 + i, std::false_type{}, ic, acc[i]);
-            // the arm differences of this plane, in the same order as a halo plane's
-            if constexpr (i == 0) {
-                spread(acz, h, 1, std::integral_constant<int, MC>{});
-            } else if constexpr (i == 1) {
-                spread(acz, gd, 2, std::integral_constant<int, MC>{});
-            } else {
-                spread(acx, h, 1, std::integral_constant<int, MC>{});
-                spread(acy, gd, 2, std::integral_constant<int, MC>{});
+                for (int a = 0; a < 3; ++a)  // advection and d_a u_i d_a lnrho
+                    acc[i] = P::fma(g[a], q[a], acc[i]);
+#pragma unroll
+                for (int a = 0; a < 3; ++a)  // d_a u_i d_i lnrho, for component a
+                    acc[a] = i == 0 && a > 0 ? P::mul(g[a], nng[0]) : P::fma(g[a], nng[i], acc[a]);
+                dvm = i == 0 ? g[0] : P::add(dvm, g[i]);
+                if constexpr (i == 0)
+                    mix_xy(1, acc[1]);  // D_xy u_x -> y
+                else if constexpr (i == 1)
+                    mix_xy(2, acc[0]);  // D_xy u_y -> x
+            };
+            component(std::integral_constant<int, 0>{});
+            component(std::integral_constant<int, 1>{});
+            component(std::integral_constant<int, 2>{});
+            if constexpr (NF == 5) {
+                axial(4, std::false_type{}, NoComp{}, acc[0]);
+                prn[4] = P::fma(uc[2], g[2], P::fma(uc[1], g[1], P::mul(uc[0], g[0])));
             }
+            const V ug = P::fma(uc[2], gl[2], P::fma(uc[1], gl[1], P::mul(uc[0], gl[0])));
+            prn[0] = P::fma(P::bc(c.ns), ug, dvm);
+            const V t = P::fma(P::bc(c.nu23), dvm, P::bc(c.ncs2));
 #pragma unroll
-            for (int a = 0; a < 3; ++a)  // advection and d_a u_i d_a lnrho
-                acc[i] = P::fma(g[a], q[a], acc[i]);
+            for (int a = 0; a < 3; ++a)
+                prn[1 + a] = P::fma(t, gl[a], acc[a]);
+        } else {
+            V g[3], d2[3], h[3], gd[3], y1p, y1m;
+            auto axial = [&](int f, bool second) {
+                const V cc = C(f, 3);
+                V m4, m2, p2, p4;
+                xnb(cb + f * FSTRIDE, cc, m4, m2, p2, p4);
+                xdiff(m4, m2, cc, p2, p4, h);
+                g[0] = P::fma(P::bc(c.D1(0, 3)), h[2],
+                              P::fma(P::bc(c.D1(0, 2)), h[1], P::mul(P::bc(c.D1(0, 1)), h[0])));
+                if (second) {
+                    const V s1 = P::mk(cc.y + m2.y, p2.x + cc.x);
+                    const V s3 = P::mk(p2.y + m4.y, p4.x + m2.x);
+                    d2[0] = P::fma(P::bc(c.D2(0, 3)), s3,
+                                   P::fma(P::bc(c.D2(0, 2)), P::add(p2, m2),
+                                          P::fma(P::bc(c.D2(0, 1)), s1, P::mul(P::bc(c.D2c(0)), cc))));
+                }
+                V gy, by, gz, bz;
 #pragma unroll
-            for (int a = 0; a < 3; ++a)  // d_a u_i d_i lnrho, for component a
-                acc[a] = i == 0 && a > 0 ? P::mul(g[a], nng[0]) : P::fma(g[a], nng[i], acc[a]);
-            dvm = i == 0 ? g[0] : P::add(dvm, g[i]);
-            if constexpr (i == 0)
-                mix_xy(1, acc[1]);  // D_xy u_x -> y
-            else if constexpr (i == 1)
-                mix_xy(2, acc[0]);  // D_xy u_y -> x
-        };
-        component(std::integral_constant<int, 0>{});
-        component(std::integral_constant<int, 1>{});
-        component(std::integral_constant<int, 2>{});
-        if constexpr (NF == 5) {
-            axial(4, std::false_type{}, NoComp{}, acc[0]);
-            prn[4] = P::fma(uc[2], g[2], P::fma(uc[1], g[1], P::mul(uc[0], g[0])));
+                for (int k = 1; k <= 3; ++k) {
+                    const V yp = ld2(f, k, 0), ym = ld2(f, -k, 0);
+                    if (k == 1) {
+                        y1p = yp;
+                        y1m = ym;
+                    }
+                    const V zp = C(f, 3 + k), zm = C(f, 3 - k);
+                    const V dyv = P::fma(ym, NEG1, yp), dzv = P::fma(zm, NEG1, zp);
+                    gd[k - 1] = dyv;
+                    gy = k == 1 ? P::mul(P::bc(c.D1(1, k)), dyv) : P::fma(P::bc(c.D1(1, k)), dyv, gy);
+                    gz = k == 1 ? P::mul(P::bc(c.D1(2, k)), dzv) : P::fma(P::bc(c.D1(2, k)), dzv, gz);
+                    if (second) {
+                        if (k == 1) {
+                            by = P::mul(P::bc(c.D2c(1)), C(f, 3));
+                            bz = P::mul(P::bc(c.D2c(2)), C(f, 3));
+                        }
+                        by = P::fma(P::bc(c.D2(1, k)), P::add(yp, ym), by);
+                        bz = P::fma(P::bc(c.D2(2, k)), P::add(zp, zm), bz);
+                    }
+                }
+                g[1] = gy;
+                g[2] = gz;
+                if (second) {
+                    d2[1] = by;
+                    d2[2] = bz;
+                }
+            };
+            // Eq. 8 in the (x, y) plane: D_xy f = sum_k MX_k [h_k(y+k) - h_k(y-k)];
+            // the centre pairs of rows y+-1 are those of the y arm just loaded
+            auto mix_xy = [&](int f) -> V {
+                V a;
+#pragma unroll
+                for (int k = 1; k <= 3; ++k) {
+                    V hh[2];
+#pragma unroll
+                    for (int sgn = 0; sgn < 2; ++sgn) {
+                        const int dy = sgn ? -k : k;
+                        const V m2 = ld2(f, dy, -2), p2 = ld2(f, dy, 2);
+                        if (k == 1) {
+                            const V cc = sgn ? y1m : y1p;
+                            hh[sgn] = P::mk(cc.y - m2.y, p2.x - cc.x);
+                        } else if (k == 2) {
+                            hh[sgn] = P::fma(m2, NEG1, p2);
+                        } else {
+                            const V m4 = ld2(f, dy, -4), p4 = ld2(f, dy, 4);
+                            hh[sgn] = P::mk(p2.y - m4.y, p4.x - m2.x);
+                        }
+                    }
+                    const V d = P::fma(hh[1], NEG1, hh[0]);
+                    a = k == 1 ? P::mul(P::bc(c.MX(0, k)), d) : P::fma(P::bc(c.MX(0, k)), d, a);
+                }
+                return a;
+            };
+            const V NU = P::bc(c.nu), NU3 = P::bc(c.nu3);
+            const V uc[3] = {C(1, 3), C(2, 3), C(3, 3)};
+            V acc[4], gl[3];
+            V dv = P::bc(0.f);
+            axial(0, false);
+            gl[0] = g[0];
+            gl[1] = g[1];
+            gl[2] = g[2];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                axial(1 + i, true);
+                // the arm differences of this plane, in the same order as a halo plane's
+                if (i == 0) {
+                    spread(acz, h, 1, std::integral_constant<int, MC>{});
+                } else if (i == 1) {
+                    spread(acz, gd, 2, std::integral_constant<int, MC>{});
+                } else {
+                    spread(acx, h, 1, std::integral_constant<int, MC>{});
+                    spread(acy, gd, 2, std::integral_constant<int, MC>{});
+                }
+                V adv = P::mul(uc[0], g[0]);
+                adv = P::fma(uc[1], g[1], adv);
+                adv = P::fma(uc[2], g[2], adv);
+                const V lap = P::add(P::add(d2[0], d2[1]), d2[2]);
+                V sg = P::mul(g[0], gl[0]);
+                sg = P::fma(g[1], gl[1], sg);
+                sg = P::fma(g[2], gl[2], sg);
+                V ai = P::mul(NU, P::add(lap, sg));
+                if (i > 0)
+                    ai = P::add(ai, acc[1 + i]);
+                ai = P::fma(adv, NEG1, ai);
+                ai = P::fma(NU3, d2[i], ai);
+                acc[1 + i] = ai;
+                const V nugl = P::mul(NU, gl[i]);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    if (a == i)
+                        acc[1 + a] = P::fma(g[a], nugl, acc[1 + a]);
+                    else if (a > i && i == 0)
+                        acc[1 + a] = P::mul(g[a], nugl);  // first contribution
+                    else
+                        acc[1 + a] = P::fma(g[a], nugl, acc[1 + a]);
+                }
+                dv = P::add(dv, g[i]);
+                if (i == 0)
+                    acc[2] = P::fma(NU3, mix_xy(1), acc[2]);  // D_xy u_x -> y
+                else if (i == 1)
+                    acc[1] = P::fma(NU3, mix_xy(2), acc[1]);  // D_xy u_y -> x
+            }
+            if constexpr (NF == 5) {
+                axial(4, false);
+                V t = P::mul(uc[0], g[0]);
+                t = P::fma(uc[1], g[1], t);
+                t = P::fma(uc[2], g[2], t);
+                prn[4] = P::mul(t, NEG1);
+            }
+            V ug = P::mul(uc[0], gl[0]);
+            ug = P::fma(uc[1], gl[1], ug);
+            ug = P::fma(uc[2], gl[2], ug);
+            prn[0] = P::mul(P::add(ug, dv), NEG1);
+            const V NCS2 = P::bc(-c.cs2);
+            const V t = P::mul(P::bc(-c.nu23), dv);
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                prn[1 + a] = P::fma(t, gl[a], P::fma(NCS2, gl[a], acc[1 + a]));
         }
-        const V ug = P::fma(uc[2], gl[2], P::fma(uc[1], gl[1], P::mul(uc[0], gl[0])));
-        prn[0] = P::fma(P::bc(c.ns), ug, dvm);
-        const V t = P::fma(P::bc(c.nu23), dvm, P::bc(c.ncs2));
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            prn[1 + a] = P::fma(t, gl[a], acc[a]);
     };
 
     // output plane o (window index S): add the z-paired terms and the
@@ -512,11 +658,18 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
 #pragma unroll
             for (int f = 0; f < NF; ++f)
                 r[f] = prv[f];
-            r[1] = P::add(r[1], acx[S]);
-            r[2] = P::add(r[2], acy[S]);
-            r[3] = P::add(r[3], acz[S]);
+            if constexpr (FOLD) {
+                r[1] = P::add(r[1], acx[S]);
+                r[2] = P::add(r[2], acy[S]);
+                r[3] = P::add(r[3], acz[S]);
+            } else {
+                const V NU3 = P::bc(c.nu3);
+                r[1] = P::fma(NU3, acx[S], r[1]);
+                r[2] = P::fma(NU3, acy[S], r[2]);
+                r[3] = P::fma(NU3, acz[S], r[3]);
+            }
             if constexpr (FORCE) {
-                // f_i = amp_i cos(k.x + phi) (amp folded like the weights)
+                // f_i = amp_i cos(k.x + phi)
                 const float2 cz = fo->tz32[z0 + o];
                 const V fc = P::mk(fxy0.x * cz.x - fxy0.y * cz.y, fxy1.x * cz.x - fxy1.y * cz.y);
 #pragma unroll
@@ -529,9 +682,15 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
                 const V u0 = colv[f][S];
                 V o2;
                 if constexpr (UP32) {
-                    // (dt is in the weights)
                     const V ALPHA = P::bc(alpha), BETA = P::bc(beta);
-                    const V wn = first ? r[f] : P::fma(ALPHA, wv[f], r[f]);
+                    V wn;
+                    if constexpr (FOLD) {  // (dt is in the weights)
+                        static_assert(!FORCE, "amp takes no dt");
+                        wn = first ? r[f] : P::fma(ALPHA, wv[f], r[f]);
+                    } else {
+                        const V DT = P::bc(dt);
+                        wn = first ? P::mul(DT, r[f]) : P::fma(DT, r[f], P::mul(ALPHA, wv[f]));
+                    }
                     o2 = P::fma(BETA, wn, u0);
                     if (!last)
                         *reinterpret_cast<V *>(w + f * Lw.fpitch + go_w) = wn;
@@ -745,8 +904,9 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
 }
 
 // Single box: one CTA per (tile, z-chunk).
-// CoefT: FoldCoef<float>, or FoldCubic<float> when the grid spacing is the same
-// on every axis (20 weights instead of 52).
+// CoefT: Coef<float>, or CubicCoef<float> when the grid spacing is the same on
+// every axis (10 stencil weights instead of 30, few enough to stay in uniform
+// registers).
 template <class TW, class TA, int NF, int TX, int TY, int NS, int U, int MINB, bool ICVT,
           bool FORCE, bool TM, class CoefT, bool SHFL, int STG = -1, bool FULL = false>
 __global__ void __launch_bounds__((TX / 2) * TY, MINB) k_substep_lag(
@@ -811,35 +971,26 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
     float *out = (float *)b.out;
     TW *w = (TW *)b.w;
     cudaError_t e = cudaErrorNotSupported;
-    // the weights with the time step folded in where the update is FP32 (the
-    // precision forms multiply by dt in their own arithmetic); equal spacing
-    // on every axis: the isotropic set (same values)
-    (void)c;
-    constexpr bool UP32 = std::is_same<TA, float>::value && std::is_same<TW, float>::value;
-    const FoldCoef<float> fc = make_fold<float>(*b.cd, UP32 ? st.dt : 1.0);
-    const bool iso = TM && fold_is_cubic(fc);
-    const FoldCubic<float> cc = cubic_of(fc);
-    RKStage sd = st;  // the forcing takes the time step too
-    if (UP32)
-        for (int a = 0; a < 3; ++a)
-            sd.fo.amp32[a] = (float)(st.fo.amp[a] * st.dt);
+    // equal spacing on every axis: the isotropic weights (same values)
+    const bool iso = TM && coef_is_cubic(c);
+    const CubicCoef<float> cc = cubic_of(c);
 #define GBFD_LAUNCH_LAG_C(NFV, FRC, CT, CV)                                                       \
     do {                                                                                          \
         constexpr auto kern = tiled4::k_substep_lag<TW, TA, NFV, TX, TY, NS, U, MINB, ICVT, FRC,  \
                                                     TM, CT, SHFL>;                                \
         constexpr int sm = tiled4::RingL<TW, NFV, TX, TY, NS, U>::BYTES;                          \
         e = launch_chained<kern>(grid, block, sm, false, stream, *map, *wmap, out, w, b.Ls, b.Lw, \
-                                 CV, sd, zc, tiles_x, dev_error, skip_plane);                     \
+                                 CV, st, zc, tiles_x, dev_error, skip_plane);                     \
     } while (0)
 #define GBFD_LAUNCH_LAG(NFV, FRC)                                                                 \
     do {                                                                                          \
         if constexpr (TM) {                                                                       \
             if (iso) {                                                                            \
-                GBFD_LAUNCH_LAG_C(NFV, FRC, FoldCubic<float>, cc);                                \
+                GBFD_LAUNCH_LAG_C(NFV, FRC, CubicCoef<float>, cc);                                \
                 break;                                                                            \
             }                                                                                     \
         }                                                                                         \
-        GBFD_LAUNCH_LAG_C(NFV, FRC, FoldCoef<float>, fc);                                              \
+        GBFD_LAUNCH_LAG_C(NFV, FRC, Coef<float>, c);                                              \
     } while (0)
     // the five-field isotropic case on whole tiles of a large grid (forced steps
     // in FP32 arithmetic included): the substep is a template argument and the
@@ -856,10 +1007,10 @@ cudaError_t launch_lag_cfg(const StateBufs &b, const Coef<float> &c, const RKSta
 #define GBFD_LAUNCH_LAG_S(FRC, SV)                                                                \
     do {                                                                                          \
         constexpr auto kern = tiled4::k_substep_lag<TW, TA, 5, TX, TY, NS, U, MINB, ICVT, FRC,    \
-                                                    TM, FoldCubic<float>, SHFL, SV, true>;        \
+                                                    TM, CubicCoef<float>, SHFL, SV, true>;        \
         constexpr int sm = tiled4::RingL<TW, 5, TX, TY, NS, U>::BYTES;                            \
         e = launch_chained<kern>(grid, block, sm, false, stream, *map, *wmap, out, w, b.Ls, b.Lw, \
-                                 cc, sd, zc, tiles_x, dev_error, skip_plane);                     \
+                                 cc, st, zc, tiles_x, dev_error, skip_plane);                     \
     } while (0)
 #define GBFD_LAUNCH_LAG_SS(FRC)                                                                   \
     do {                                                                                          \

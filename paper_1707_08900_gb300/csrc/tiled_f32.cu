@@ -40,7 +40,7 @@ cudaError_t launch_substep_tiled(const StateBufs &b, const Coef<TS> &c, const RK
     } else if (v == kVarLagTm) {
         const bool whole = b.Ls.nx % 32 == 0 && b.Ls.ny % 8 == 0 && nf == 5 && coef_is_cubic(c);
         if (!st.fo.on && !whole && stage_kernels(b.Ls) && st.s >= 0 && st.s <= 2)
-            e = launch_lag_stage(b, st, nf, t.zc, v, dev_error, cache, stream, launches);
+            e = launch_lag_stage(b, c, st, nf, t.zc, v, dev_error, cache, stream, launches);
         else
             e = launch_lag_cfg<TW, TA, 32, 8, 8, 2, true>(b, c, st, nf, t.zc, v, dev_error, cache,
                                                         stream, launches);

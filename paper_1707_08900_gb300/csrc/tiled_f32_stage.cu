@@ -37,21 +37,21 @@ cudaError_t launch_s(const StateBufs &b, const CoefT &c, const RKStage &st, int 
 
 }  // namespace
 
-cudaError_t launch_lag_stage(const StateBufs &b, const RKStage &st, int nf, int zc, int cfg_key,
-                             int *dev_error, TmapCache *cache, cudaStream_t stream, int *launches)
+cudaError_t launch_lag_stage(const StateBufs &b, const Coef<float> &c, const RKStage &st, int nf,
+                             int zc, int cfg_key, int *dev_error, TmapCache *cache,
+                             cudaStream_t stream, int *launches)
 {
     CUtensorMap *map = nullptr, *wmap = nullptr;
     if (!get_state_tmap(cache, b.in, b.Ls, nf, 32, 8, cfg_key, &map) ||
         !get_tile_tmap(cache, b.w, b.Lw, nf, 32, 8, cfg_key, &wmap))
         return cudaErrorInvalidValue;
-    const FoldCoef<float> fc = make_fold<float>(*b.cd, st.dt);
-    const bool iso = fold_is_cubic(fc);
+    const bool iso = coef_is_cubic(c);
     *launches += 1;
     if (nf == 5)
-        return iso ? launch_s<5>(b, cubic_of(fc), st, zc, dev_error, *map, *wmap, stream)
-                   : launch_s<5>(b, fc, st, zc, dev_error, *map, *wmap, stream);
-    return iso ? launch_s<4>(b, cubic_of(fc), st, zc, dev_error, *map, *wmap, stream)
-               : launch_s<4>(b, fc, st, zc, dev_error, *map, *wmap, stream);
+        return iso ? launch_s<5>(b, cubic_of(c), st, zc, dev_error, *map, *wmap, stream)
+                   : launch_s<5>(b, c, st, zc, dev_error, *map, *wmap, stream);
+    return iso ? launch_s<4>(b, cubic_of(c), st, zc, dev_error, *map, *wmap, stream)
+               : launch_s<4>(b, c, st, zc, dev_error, *map, *wmap, stream);
 }
 
 }  // namespace gbfd
