@@ -64,7 +64,7 @@ struct BoxDesc {
 // What a step's time steps make of each box, refreshed before every replay.
 struct BoxStep {
     float dt;
-    FoldCubic<float> fold;  // the lagged routine's weights, dt folded in
+    FoldAxes fold;  // the lagged routine's weights, dt folded in
 };
 
 // Device-side state of the dataflow launch, zeroed before each launch.
@@ -91,7 +91,7 @@ constexpr int smem_bytes()
 template <int KIND, int NF, bool SPEC = false>
 __device__ __forceinline__ bool run_item(const BoxDesc *__restrict__ B, const int4 item,
                                          const int s, const int parity, const float dt,
-                                         const int zc, const FoldCubic<float> &scoef, int &jrun,
+                                         const int zc, const FoldAxes &scoef, int &jrun,
                                          int &wrun, unsigned char *smem, int *dev_error,
                                          const uint32_t tmem)
 {
@@ -109,7 +109,7 @@ __device__ __forceinline__ bool run_item(const BoxDesc *__restrict__ B, const in
                 auto run = [&](auto stg) {
                     constexpr int S = decltype(stg)::value;
                     return tiled4::run_column<float, float, NF, TX, TY, NS, U, false, false, true,
-                                              FoldCubic<float>, false, S, true>(
+                                              FoldAxes, false, S, true>(
                         &B->tm_state[wi][parity], &B->tm_w[wi], B->state[parity ^ 1], B->w, L, L,
                         scoef, alpha, beta, dt, S == 0, S == 2, item.y, item.z, item.w, nout, jrun,
                         wrun, smem, dev_error, -1, nullptr, tmem);
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__((kind_tx(KIND) / 2) * TY) k_batch_substep(
 {
     constexpr int SMB = smem_bytes<KIND, NF>();
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ FoldCubic<float> scoef;
+    __shared__ FoldAxes scoef;
     if constexpr (KIND == KIND_LAG)
         tiled2::init_barriers(reinterpret_cast<uint64_t *>(
                                   smem + tiled4::RingL<float, NF, 32, TY, NS, U>::BAR_OFF),
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__((kind_tx(KIND) / 2) * TY) k_batch_flow(
 {
     constexpr int SMB = smem_bytes<KIND, NF>();
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ FoldCubic<float> scoef;
+    __shared__ FoldAxes scoef;
     __shared__ int sq;
     if constexpr (KIND == KIND_LAG)
         tiled2::init_barriers(reinterpret_cast<uint64_t *>(
@@ -674,7 +674,7 @@ cudaError_t upload_steps(gbfd_batch *b, const double *dt)
     for (int i = 0; i < b->nbox; ++i) {
         const double d = dt ? dt[i] : 0.0;
         h[i].dt = (float)d;
-        h[i].fold = cubic_of(make_fold<float>(b->hcoef[i], d));
+        h[i].fold = make_fold_axes(b->hcoef[i], d);
     }
     cudaError_t e = cudaMemcpyAsync(b->dstep, h.data(), sizeof(BoxStep) * b->nbox,
                                     cudaMemcpyHostToDevice, b->stream);

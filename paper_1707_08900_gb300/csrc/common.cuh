@@ -199,7 +199,7 @@ inline CubicCoef<T> make_cubic_coef(double h, double cs, double nu)
     return q;
 }
 
-// Weights of the lagged kernels with everything that multiplies a linear term
+// Weights of the FP64 lagged kernel with everything that multiplies a linear term
 // folded in: the time step s (1 where the update multiplies by dt itself), the
 // viscosity and the signs.  With gm = -s grad u (weights N1) and nng = -nu
 // grad lnrho, Eqs. 1-3 of component i become
@@ -213,8 +213,7 @@ inline CubicCoef<T> make_cubic_coef(double h, double cs, double nu)
 // they cancel on a constant as they do in Eq. 7; the arms X2 take what rounding
 // VC left over, the first arm as much of it as its last bit shows, the next ones
 // the rest (no arm moves by more than about one unit of the first one's last
-// place).  Left over, it adds the same multiple of u in every substep: up to
-// 3e-8 per step at VC = 0.9 in FP32, 3e-7 of a mean flow after ten steps.
+// place).  Left over, it adds the same multiple of u in every substep.
 template <class T>
 struct FoldCoef {
     T l1[3][3];  // d1
@@ -245,12 +244,58 @@ struct FoldCubic {
     __host__ __device__ __forceinline__ T M3(int, int k) const { return m3[k - 1]; }
 };
 
+// The batch's FP32 form of the folding, for equal spacing: every axis has a centre
+// weight of its own (cx beside X2, cv beside V2), so that each axis' sum cancels
+// by itself before the three are added.  In one sum with the common centre weight
+// VC the partial sums round against VC u until the last arm: at the viscous limit
+// of the time step (VC = 2.3) two FP32 steps were 2.1e-7 off (rms of the velocity at
+// 20^3 to 48^3) where the two-plane routine's separate second derivatives, which
+// these now are, leave 1.2e-7.
+struct FoldAxes {
+    float l1[3], n1[3], v2[3], x2[3], cv, cx, m3[3];
+    float nnu, nu23, ncs2, ns;
+    __host__ __device__ __forceinline__ float L1(int, int k) const { return l1[k - 1]; }
+    __host__ __device__ __forceinline__ float N1(int, int k) const { return n1[k - 1]; }
+    __host__ __device__ __forceinline__ float V2(int, int k) const { return v2[k - 1]; }
+    __host__ __device__ __forceinline__ float X2(int, int k) const { return x2[k - 1]; }
+    __host__ __device__ __forceinline__ float M3(int, int k) const { return m3[k - 1]; }
+};
+
 template <class C>
-struct is_fold : std::false_type {};
-template <class T>
-struct is_fold<FoldCoef<T>> : std::true_type {};
-template <class T>
-struct is_fold<FoldCubic<T>> : std::true_type {};
+struct is_fold : std::is_same<C, FoldAxes> {};
+
+// Centre weight of the arms w, which take what its rounding left over (as above).
+inline float centre_of(float (&w)[3])
+{
+    const double sum = 2.0 * ((double)w[0] + ((double)w[1] + (double)w[2]));
+    const float c = (float)(-sum);
+    double left = (double)c + sum;  // exact: 24-bit terms of few binades apart
+    for (int k = 0; k < 3; ++k) {
+        const float arm = (float)((double)w[k] - 0.5 * left);
+        left += 2.0 * ((double)arm - (double)w[k]);
+        w[k] = arm;
+    }
+    return c;
+}
+
+inline FoldAxes make_fold_axes(const Coef<double> &c, double s)
+{
+    FoldAxes f;
+    for (int k = 0; k < 3; ++k) {
+        f.l1[k] = (float)c.d1[0][k];
+        f.n1[k] = (float)(-s * c.d1[0][k]);
+        f.v2[k] = (float)(s * c.nu * c.d2[0][k]);
+        f.x2[k] = (float)(s * c.nu * (4.0 / 3.0) * c.d2[0][k]);
+        f.m3[k] = (float)(s * (c.nu / 3.0) * c.mx[0][k]);
+    }
+    f.cv = centre_of(f.v2);
+    f.cx = centre_of(f.x2);
+    f.nnu = (float)(-c.nu);
+    f.nu23 = (float)(2.0 * c.nu / 3.0);
+    f.ncs2 = (float)(-s * c.cs2);
+    f.ns = (float)(-s);
+    return f;
+}
 
 template <class T>
 inline FoldCoef<T> make_fold(const Coef<double> &c, double s)

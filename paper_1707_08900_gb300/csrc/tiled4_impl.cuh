@@ -22,12 +22,10 @@
 // three halo planes below and above a z-chunk are never centres: their arm
 // differences come from loads of their own.
 //
-// With folded weights (FoldCoef, common.cuh; the batch's lagged routine) every
-// derivative goes straight into the right-hand side: 3% faster at 256^3 (3.40 and
-// 3.30 ms for four steps).  The single box does not take them: all terms round
-// against the largest one, VC u, which grows with nu dt / h^2, and at 512^3 two
-// steps are 7.5e-8 from the 64-bit result instead of 6.0e-8; the batch's boxes are
-// small (VC below 0.4) and as near with either (6.7e-8).
+// With folded weights (FoldAxes, common.cuh; the batch's lagged routine) every
+// derivative goes straight into the right-hand side, the second derivatives as one
+// cancelling sum per axis.  The single box does not take them: its arithmetic is
+// the one that corrected runs were trained and are compared with.
 //
 // Per output plane and thread this reads 92 shared pairs (5 column values,
 // 50 x/y arms of the five fields, 32 for the two (x, y) cross terms, 5 of
@@ -377,18 +375,20 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
                 constexpr int I = decltype(ic)::value;
                 auto w1 = [&](int a, int k) { return P::bc(LN ? c.L1(a, k) : c.N1(a, k)); };
                 auto w2 = [&](int a, int k) { return P::bc(a == I ? c.X2(a, k) : c.V2(a, k)); };
+                auto wc = [&](int a) { return P::bc(a == I ? c.cx : c.cv); };
                 const V cc = C(f, 3);
                 V m4, m2, p2, p4;
                 xnb(cb + f * FSTRIDE, cc, m4, m2, p2, p4);
                 xdiff(m4, m2, cc, p2, p4, h);
                 g[0] = P::fma(w1(0, 3), h[2], P::fma(w1(0, 2), h[1], P::mul(w1(0, 1), h[0])));
+                V bx, by, bz;
                 if constexpr (I >= 0) {
                     const V s1 = P::mk(cc.y + m2.y, p2.x + cc.x);
                     const V s3 = P::mk(p2.y + m4.y, p4.x + m2.x);
-                    acc = P::fma(w2(0, 3), s3,
-                                 P::fma(w2(0, 2), P::add(p2, m2), P::fma(w2(0, 1), s1, acc)));
+                    bx = P::fma(w2(0, 3), s3,
+                                P::fma(w2(0, 2), P::add(p2, m2),
+                                       P::fma(w2(0, 1), s1, P::mul(wc(0), cc))));
                 }
-                V byz;
 #pragma unroll
                 for (int k = 1; k <= 3; ++k) {
                     const V yp = ld2(f, k, 0), ym = ld2(f, -k, 0);
@@ -402,13 +402,18 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
                     g[1] = k == 1 ? P::mul(w1(1, 1), dyv) : P::fma(w1(1, k), dyv, g[1]);
                     g[2] = k == 1 ? P::mul(w1(2, 1), dzv) : P::fma(w1(2, k), dzv, g[2]);
                     if constexpr (I >= 0) {
-                        byz = k == 1 ? P::mul(w2(1, 1), P::add(yp, ym))
-                                     : P::fma(w2(1, k), P::add(yp, ym), byz);
-                        byz = P::fma(w2(2, k), P::add(zp, zm), byz);
+                        if (k == 1) {
+                            by = P::mul(wc(1), cc);
+                            bz = P::mul(wc(2), cc);
+                        }
+                        by = P::fma(w2(1, k), P::add(yp, ym), by);
+                        bz = P::fma(w2(2, k), P::add(zp, zm), bz);
                     }
                 }
-                if constexpr (I >= 0)
-                    acc = P::add(acc, byz);
+                if constexpr (I >= 0) {
+                    const V b = P::add(P::add(bx, by), bz);
+                    acc = I == 0 ? b : P::add(acc, b);  // component 0 begins its sum here
+                }
             };
             // Eq. 8 in the (x, y) plane, onto acc: D_xy f = sum_k MX_k [h_k(y+k) -
             // h_k(y-k)]; the centre pairs of rows y+-1 are those of the y arm just
@@ -447,8 +452,6 @@ __device__ __forceinline__ bool run_column(const CUtensorMap *tmap, const CUtens
             }
             auto component = [&](auto ic) {
                 constexpr int i = decltype(ic)::value;
-                acc[i] = i == 0 ? P::mul(P::bc(c.VC(0)), uc[0])
-                                : P::fma(P::bc(c.VC(i)), uc[i], acc[i]);
                 axial(1 + i, std::false_type{}, ic, acc[i]);
                 // the arm differences of this plane, in the same order as a halo plane's
                 if constexpr (i == 0) {
