@@ -773,6 +773,10 @@ __global__ void __launch_bounds__(256) k_loss(const float *y, const float *__res
     chain_next();
     const int n3 = n * n * n;
     __shared__ double sh[256];
+    // of channel c at element i of the states, y the network's output there
+    auto residual = [&](float yc, int c, long long i) {
+        return yc - (c < nf ? (ts[i] - xs[i]) / sout[c] : 0.f);
+    };
     float hi = 0.f, lo = 0.f;
 #pragma unroll
     for (int k = 0; k < LOSS_PTS; ++k) {
@@ -788,9 +792,7 @@ __global__ void __launch_bounds__(256) k_loss(const float *y, const float *__res
             d[c] = 0.f;
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            const long long i = ((long long)b * NC + c) * n3 + r;
-            const float t = c < nf ? (ts[i] - xs[i]) / sout[c] : 0.f;
-            const float e = yv[c] - t;
+            const float e = residual(yv[c], c, ((long long)b * NC + c) * n3 + r);
             float sq, err, sum, rest;
             two_prod(e, e, sq, err);
             two_sum(hi, sq, sum, rest);
@@ -801,8 +803,24 @@ __global__ void __launch_bounds__(256) k_loss(const float *y, const float *__res
         // dY3 into the padded chunk-major layout, with its periodic copies
         put_chunk0(dy3, d, b, r % n, (r / n) % n, r / (n * n), n, B);
     }
-    // (an overflowing or undefined sum has no error term)
-    sh[threadIdx.x] = isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+    double sum = (double)hi + (double)lo;
+    if (!(hi >= 0x1p-100f && hi < INFINITY)) {
+        // squares or their error terms outside the FP32 range: again in FP64
+        sum = 0.0;
+#pragma unroll 1
+        for (int k = 0; k < LOSS_PTS; ++k) {
+            const int p = (blockIdx.x * LOSS_PTS + k) * 256 + threadIdx.x;
+            if (p >= npts)
+                break;
+            const int b = p / n3, r = p - b * n3;
+#pragma unroll 1
+            for (int c = 0; c < NC; ++c) {
+                const double e = residual(y[(long long)p * 8 + c], c, ((long long)b * NC + c) * n3 + r);
+                sum += e * e;
+            }
+        }
+    }
+    sh[threadIdx.x] = sum;
     __syncthreads();
     for (int s = 128; s > 0; s >>= 1) {
         if (threadIdx.x < s)
