@@ -24,26 +24,25 @@ __device__ __forceinline__ void chain_next()
 }
 
 // Launch of KERN in the chain; its shared-memory limit (and, with `carveout`,
-// its preference for shared memory over L1) is set once per device.
+// its preference for shared memory over L1) is set once per device (the runtime
+// keeps it with the function, through a device reset and in other contexts).
 template <auto KERN, class... Args>
 cudaError_t launch_chained(dim3 grid, dim3 block, int smem, bool carveout, cudaStream_t stream,
                            Args... args)
 {
     static std::atomic<unsigned long long> opted{0};
+    cudaError_t e = cudaSuccess;
     if (smem > 0) {
         int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess)
-            return e;
-        const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
-        if (!(opted.load() & bit)) {
+        e = cudaGetDevice(&dev);
+        const unsigned long long bit = e == cudaSuccess && dev < 64 ? 1ull << dev : 0;
+        if (e == cudaSuccess && !(opted.load() & bit)) {
             e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e == cudaSuccess && carveout)
                 e = cudaFuncSetAttribute(KERN, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          (int)cudaSharedmemCarveoutMaxShared);
-            if (e != cudaSuccess)
-                return e;
-            opted.fetch_or(bit);
+            if (e == cudaSuccess)
+                opted.fetch_or(bit);
         }
     }
     cudaLaunchConfig_t cfg = {};
@@ -56,7 +55,11 @@ cudaError_t launch_chained(dim3 grid, dim3 block, int smem, bool carveout, cudaS
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, KERN, args...);
+    if (e == cudaSuccess)
+        e = cudaLaunchKernelEx(&cfg, KERN, args...);
+    if (e != cudaSuccess)
+        (void)cudaGetLastError();  // reported by the caller, not left for its next launch
+    return e;
 }
 
 // The body force f of Eq. 2 for the current time step: the non-helical
