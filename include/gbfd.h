@@ -268,8 +268,9 @@ gbfd_status gbfd_tc_mma_cycles(int n, void *stream, double *cycles);
 
 /* Tuning options (no counterpart in the paper; used by the tests and the
  * autotuner).  GBFD_OPT_KERNEL_PATH: 0 = tiled kernels (TMA-staged shared
- * memory, the default), 1 = simple one-thread-per-point kernels reading
- * global memory.  GBFD_OPT_TILE_CONFIG: index into the tiled kernels' tile
+ * memory), 1 = simple one-thread-per-point kernels reading global memory; until
+ * it is set, the tiled kernels except for the FP64 19-point form, which runs
+ * the simple ones.  GBFD_OPT_TILE_CONFIG: index into the tiled kernels' tile
  * table, -1 = built-in default.  Out-of-range values -> INVALID_ARG. */
 enum {
     GBFD_OPT_KERNEL_PATH = 1,

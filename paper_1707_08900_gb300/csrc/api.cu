@@ -36,7 +36,7 @@ struct gbfd_ctx {
     int ndiag;
     int cur;         // which state buffer holds the current state
     int64_t launches;
-    int kernel_path;  // 0 = tiled when supported, 1 = simple
+    int kernel_path;  // -1 = unset (run_tiled chooses), 0 = tiled, 1 = simple
     int tile_cfg;     // index into the tiled kernel's tile table (-1 = default)
     int zc;           // planes per CTA of the default tiled kernel (default_zc)
     double h[3];      // grid spacings (z: lz / (nz - 1) between walls)
@@ -269,6 +269,17 @@ bool write_cache(const char *path, const std::map<std::string, std::pair<int, do
     return rename(tmp.c_str(), path) == 0;
 }
 
+// Tiled or simple kernels.  Unless the caller set the path or a tile table entry, the
+// FP64 19-point form runs the simple ones at every size: its first pass has no cross
+// terms, and one thread per point fills the FP64 pipe without halo planes (substep
+// at 32^3 27 us, tiled 30 at its best chunk; 64^3 135 and 157; 128^3 986 and 1043).
+bool run_tiled(const gbfd_ctx *c)
+{
+    if (c->kernel_path >= 0)
+        return c->kernel_path == 0;
+    return !(c->p.precision == GBFD_FP64 && c->p.form == GBFD_19P && c->tile_cfg < 0);
+}
+
 gbfd_status do_substep(gbfd_ctx *c, int s, double dt)
 {
     StateBufs b = bufs(c);
@@ -277,7 +288,7 @@ gbfd_status do_substep(gbfd_ctx *c, int s, double dt)
     st.fo = c->fo;
     int n = 0;
     cudaError_t e = cudaSuccess;
-    const bool tiled = c->kernel_path == 0;
+    const bool tiled = run_tiled(c);
     switch (c->p.precision) {
     case GBFD_FP64:
         e = tiled ? launch_substep_tiled<double, double, double>(b, c->c64, st, c->nf, c->p.form,
@@ -419,7 +430,7 @@ gbfd_status gbfd_init(const gbfd_params *p, void *workspace, size_t workspace_by
     c->ndiag = pl.ndiag;
     c->cur = 0;
     c->launches = 0;
-    c->kernel_path = 0;
+    c->kernel_path = -1;
     c->tile_cfg = -1;
     {
         // the device current at init is the context's device

@@ -7,7 +7,7 @@
 // planes behind the in-plane work (tiled6_impl.cuh) on 16 x 8 tiles, a
 // 5-slot ring, three CTAs per SM.  Forced steps (Sect. 6 forcing) of
 // variants 1-4 run variant 0 (which has the forcing term); the 19-point form
-// of variant 5 runs variant 1 (by default: the untiled kernel).
+// of variant 5 runs variant 1.
 #include "tiled6_impl.cuh"
 
 namespace gbfd {
@@ -17,12 +17,6 @@ cudaError_t launch_substep_tiled(const StateBufs &b, const Coef<TS> &c, const RK
                                  int form, int cfg, int *dev_error, TmapCache *cache,
                                  cudaStream_t stream, int *launches)
 {
-    // the 19-point form's default is the untiled kernel at every size: its first
-    // pass has no cross terms, and one thread per point fills the FP64 pipe
-    // without halo planes (substep at 32^3 27 us, tiled 30 at its best chunk;
-    // 64^3 135 and 157; 128^3 986 and 1043)
-    if (form != 0 && cfg < 0)
-        return launch_substep_simple<TS, TW, TA>(b, c, st, nf, form, stream, launches);
     const int idx = cfg < 0 ? kDefaultF64 : cfg;
     TileConfig t = tiled_config(8, idx);
     if (cfg < 0)
