@@ -271,7 +271,8 @@ gbfd_status gbfd_tc_mma_cycles(int n, void *stream, double *cycles);
  * memory), 1 = simple one-thread-per-point kernels reading global memory; until
  * it is set, the tiled kernels except for the FP64 19-point form, which runs
  * the simple ones.  GBFD_OPT_TILE_CONFIG: index into the tiled kernels' tile
- * table, -1 = built-in default.  Out-of-range values -> INVALID_ARG. */
+ * table, -1 or the index after the last = built-in default.  Out-of-range
+ * values -> INVALID_ARG. */
 enum {
     GBFD_OPT_KERNEL_PATH = 1,
     GBFD_OPT_TILE_CONFIG = 2,
@@ -297,14 +298,15 @@ enum {
 gbfd_status gbfd_set_option(gbfd_ctx *ctx, int key, int64_t value);
 
 /* Tile autotuner (no counterpart in the paper; the paper tuned block shapes
- * and points per thread by hand, Sect. 5).  Times every entry of the tiled
- * kernels' tile table on the context's current state for `reps` RK3 steps
- * each and selects the fastest; the state is not advanced (the timed
- * substeps write the spare buffer and u-tilde only).  With a non-NULL
+ * and points per thread by hand, Sect. 5).  Times the built-in default and
+ * every entry of the tiled kernels' tile table on the context's current state
+ * for `reps` RK3 steps each and selects the fastest; the state is not advanced
+ * (the timed substeps write the spare buffer and u-tilde only).  With a non-NULL
  * `cache_path`, a JSON file keyed by GPU name, grid, precision, form and
  * field count is read first (a hit skips the timing) and updated after.
- * Outputs (may be NULL): the chosen table index and its ms per RK3 step
- * (0 on a cache hit).  Synchronises the stream. */
+ * Outputs (may be NULL): the chosen table index (the one after the last for the
+ * built-in default) and its ms per RK3 step (0 on a cache hit).  Synchronises
+ * the stream. */
 gbfd_status gbfd_autotune(gbfd_ctx *ctx, int reps, const char *cache_path, int *best_cfg,
                           double *best_ms);
 

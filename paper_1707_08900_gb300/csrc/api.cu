@@ -503,9 +503,10 @@ gbfd_status gbfd_set_option(gbfd_ctx *ctx, int key, int64_t value)
         ctx->fault_skip = (int)value;
         return GBFD_OK;
     case GBFD_OPT_TILE_CONFIG:
-        if (value < -1 || value >= tiled_config_count(ctx->sbytes))
+        // (the entry after the last stands for the built-in default, as -1 does)
+        if (value < -1 || value > tiled_config_count(ctx->sbytes))
             break;
-        ctx->tile_cfg = (int)value;
+        ctx->tile_cfg = value == tiled_config_count(ctx->sbytes) ? -1 : (int)value;
         return GBFD_OK;
     default:
         break;
@@ -846,8 +847,9 @@ gbfd_status gbfd_autotune(gbfd_ctx *ctx, int reps, const char *cache_path, int *
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "autotune device query");
     char key[512];
-    snprintf(key, sizeof key, "%s|%dx%dx%d|precision%d|form%d|fields%d", prop.name, ctx->p.nx,
-             ctx->p.ny, ctx->p.nz, ctx->p.precision, ctx->p.form, ctx->nf);
+    // (table2: choices made before the default was a candidate are not read)
+    snprintf(key, sizeof key, "%s|%dx%dx%d|precision%d|form%d|fields%d|table2", prop.name,
+             ctx->p.nx, ctx->p.ny, ctx->p.nz, ctx->p.precision, ctx->p.form, ctx->nf);
     for (char *p = key; *p; ++p)
         if (*p == '"' || *p == '\\')
             *p = '_';
@@ -857,15 +859,22 @@ gbfd_status gbfd_autotune(gbfd_ctx *ctx, int reps, const char *cache_path, int *
     // the float-float form runs one kernel: tune its chunk length only
     const bool ff = ctx->p.precision == GBFD_FP32_ACCFF;
     const int count = acc ? 3 * kZcChoices : (ff ? kZcChoices : tiled_config_count(ctx->sbytes));
+    // the built-in default has kernels and chunk lengths that no entry has; its
+    // index is the one after the whole table
+    const int dflt = tiled_config_count(ctx->sbytes);
+    auto select = [&](int cfg) {
+        ctx->tile_cfg = cfg == dflt ? -1 : cfg;
+        ctx->kernel_path = cfg == dflt ? -1 : 0;
+    };
     std::map<std::string, std::pair<int, double>> cache;
     if (cache_path) {
         cache = read_cache(cache_path);
         auto it = cache.find(key);
-        if (it != cache.end() && it->second.first >= 0 && it->second.first < count) {
-            ctx->tile_cfg = it->second.first;
-            ctx->kernel_path = 0;
+        if (it != cache.end() && it->second.first >= 0 &&
+            (it->second.first < count || it->second.first == dflt)) {
+            select(it->second.first);
             if (best_cfg)
-                *best_cfg = ctx->tile_cfg;
+                *best_cfg = it->second.first;
             if (best_ms)
                 *best_ms = 0.0;
             return GBFD_OK;
@@ -879,11 +888,11 @@ gbfd_status gbfd_autotune(gbfd_ctx *ctx, int reps, const char *cache_path, int *
         return cuda_fail(ctx, e, "autotune events");
     }
     const int saved_path = ctx->kernel_path, saved_cfg = ctx->tile_cfg;
-    ctx->kernel_path = 0;
     int best = -1;
     double bms = 1e300;
-    for (int cfg = 0; cfg < count && st == GBFD_OK; ++cfg) {
-        ctx->tile_cfg = cfg;
+    for (int i = 0; i <= count && st == GBFD_OK; ++i) {
+        const int cfg = i == 0 ? dflt : i - 1;
+        select(cfg);
         for (int r = 0; r <= reps && st == GBFD_OK; ++r) {
             if (r == 1 && (e = cudaEventRecord(e0, ctx->stream)) != cudaSuccess)
                 break;
@@ -911,7 +920,7 @@ gbfd_status gbfd_autotune(gbfd_ctx *ctx, int reps, const char *cache_path, int *
         ctx->tile_cfg = saved_cfg;
         return st != GBFD_OK ? st : GBFD_ERR_CUDA;
     }
-    ctx->tile_cfg = best;
+    select(best);
     if (cache_path) {
         cache[key] = std::make_pair(best, bms);
         if (!write_cache(cache_path, cache)) {
