@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "../../include/gbfd.h"
+#include "gelu.cuh"
 #include "kernels.cuh"
 #include "tcgen05.cuh"
 #include "tiled_impl.cuh"
@@ -79,55 +80,6 @@ constexpr int kRealParams = (CH * NC * 27 + CH) + (CH * CH * 27 + CH) + (NC * CH
 __host__ __device__ inline int core_idx(int n, int k, int K)
 {
     return (n / 8) * (K * 8) + (k / 8) * 64 + (n % 8) * 8 + (k % 8);
-}
-
-// Exact GELU h Phi(h).  By erff: the polynomial below is as exact and takes 13
-// instead of 45 instructions (five corrected 64^3 steps 455 us against 470 us), but
-// moves activations across a BF16 rounding now and then, which corrected runs
-// amplify to 1e-4 of the state within eight steps.
-__device__ __forceinline__ float gelu(float h)
-{
-    return 0.5f * h * (1.0f + erff(h * 0.70710678118654752f));
-}
-__device__ __forceinline__ float2 gelu2(const float2 h) { return make_float2(gelu(h.x), gelu(h.y)); }
-
-// Its derivative Phi(h) + h phi(h), two values at a time in packed FP32x2
-// arithmetic.  With x = |h| and t = 1 / (1 + p x),
-//   1 - Phi(x) = exp(-x^2 / 2) t P(t),
-// P a degree-7 polynomial fitted here to the complementary error function
-// (minimax in relative error over 0 <= x <= 13.5, p chosen with it: 1.1e-7).
-// In FP32, max |error| of h Phi(h) over |h| <= 9 is 3.8e-7 (4.5e-7 by erff) and the
-// negative tail keeps its relative accuracy (1e-6 at h > -4, 5e-4 by 1 + erff).
-// About 13 instructions per value where erff and the rest take 45: the
-// epilogues' issue slots bound the convolutions together with the MMAs.
-struct Phi2 {
-    float2 phi, dens;  // Phi(h), exp(-h^2 / 2)
-};
-__device__ __forceinline__ Phi2 phi2(const float2 h)
-{
-    const float2 x = make_float2(fabsf(h.x), fabsf(h.y));
-    auto bc = [](float v) { return make_float2(v, v); };
-    const float2 den = __ffma2_rn(bc(0.235f), x, bc(1.f));
-    const float2 t = make_float2(__fdividef(1.f, den.x), __fdividef(1.f, den.y));
-    const float2 a = __fmul2_rn(__fmul2_rn(x, x), bc(-0.72134752f));  // log2(e) / 2
-    Phi2 r;
-    r.dens = make_float2(exp2f(a.x), exp2f(a.y));
-    float2 p = bc(-0.0640975162f);
-    p = __ffma2_rn(p, t, bc(0.209975779f));
-    p = __ffma2_rn(p, t, bc(-0.145442292f));
-    p = __ffma2_rn(p, t, bc(0.179566205f));
-    p = __ffma2_rn(p, t, bc(0.0356354676f));
-    p = __ffma2_rn(p, t, bc(0.0979318768f));
-    p = __ffma2_rn(p, t, bc(0.0926214978f));
-    p = __ffma2_rn(p, t, bc(0.0938089192f));
-    const float2 q = __fmul2_rn(r.dens, __fmul2_rn(p, t));
-    r.phi = make_float2(h.x >= 0.f ? 1.f - q.x : q.x, h.y >= 0.f ? 1.f - q.y : q.y);
-    return r;
-}
-__device__ __forceinline__ float2 gelu_grad2(const float2 h)
-{
-    const Phi2 r = phi2(h);
-    return __ffma2_rn(__fmul2_rn(h, make_float2(0.39894228f, 0.39894228f)), r.dens, r.phi);
 }
 
 // Activations live in a padded, chunk-major layout: act[c8][b][zp][yp][xp][8]
@@ -582,17 +534,15 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                                 }
 #pragma unroll
                                 for (int j = 0; j < 4; ++j)
-                                    h[j] = gelu2(h[j]);
+                                    h[j] = make_float2(gelu(h[j].x), gelu(h[j].y));
                             } else {
                                 const float4 h0 = hv[c / 4], h1 = hv[c / 4 + 1];
-                                h[0] = gelu_grad2(make_float2(h0.x, h0.y));
-                                h[1] = gelu_grad2(make_float2(h0.z, h0.w));
-                                h[2] = gelu_grad2(make_float2(h1.x, h1.y));
-                                h[3] = gelu_grad2(make_float2(h1.z, h1.w));
+                                const float hs[8] = {h0.x, h0.y, h0.z, h0.w,
+                                                     h1.x, h1.y, h1.z, h1.w};
 #pragma unroll
                                 for (int j = 0; j < 4; ++j)
-                                    h[j] = __fmul2_rn(make_float2(v[c + 2 * j], v[c + 2 * j + 1]),
-                                                      h[j]);
+                                    h[j] = make_float2(v[c + 2 * j] * gelu_grad(hs[2 * j]),
+                                                       v[c + 2 * j + 1] * gelu_grad(hs[2 * j + 1]));
                             }
                             __nv_bfloat162 w[4];
 #pragma unroll
