@@ -3,6 +3,7 @@
 // coefficients and the per-point right-hand side of Eqs. 1-3.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <type_traits>
 
@@ -491,12 +492,21 @@ __device__ __forceinline__ void rk3_update<ffloat, float, float>(bool first, ffl
 }
 
 // The FP64 update of Eq. 10 (FP32 storage) reached through float-float
-// arithmetic: carries the coefficient in both forms.
+// arithmetic: carries the coefficient in both forms.  Below 2^-100 the low half
+// runs into the subnormals and the pair no longer holds the value to 48 bits: an
+// infinite high half then makes every result fail rk3_pair_ff's check, so that
+// all take the FP64 update.
 struct fexact {
     ffloat f;
     double d;
     __host__ __device__ fexact() : d(0.0) {}
-    __host__ __device__ fexact(double v) : f(v), d(v) {}
+    __host__ __device__ fexact(double v) : f(v), d(v)
+    {
+        if (v != 0.0 && fabs(v) < 0x1p-100) {
+            f.hi = INFINITY;
+            f.lo = 0.f;
+        }
+    }
 };
 
 // Exact IEEE-754 conversions between binary32 and binary64 done with integer
