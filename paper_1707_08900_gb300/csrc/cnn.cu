@@ -632,10 +632,10 @@ __device__ __forceinline__ void put_chunk0(bf16 *dst, const float (&v)[8], int b
 }
 
 // Layer-1 input, normalised, from compact FP32 states [batch][5][n^3] (nf fields
-// present).
-__global__ void k_input_compact(const float *__restrict__ xs, int nf, int n, int npts, int B,
-                                const float *__restrict__ mean, const float *__restrict__ stdv,
-                                bf16 *__restrict__ x0)
+// present).  (Chained kernels read plainly: a read-only load could take the data
+// before the wait, while the caller's kernel still writes it.)
+__global__ void k_input_compact(const float *xs, int nf, int n, int npts, int B, const float *mean,
+                                const float *stdv, bf16 *__restrict__ x0)
 {
     // only then may the first convolution start its prologue, which reads the
     // weights that the kernel before this one may have written
@@ -654,9 +654,8 @@ __global__ void k_input_compact(const float *__restrict__ xs, int nf, int n, int
 }
 
 // Same from a solver context's padded FP32 state (one box, batch 1).
-__global__ void k_input_state(const float *st, Layout L, int nf, int B,
-                              const float *__restrict__ mean, const float *__restrict__ stdv,
-                              bf16 *__restrict__ x0)
+__global__ void k_input_state(const float *st, Layout L, int nf, int B, const float *mean,
+                              const float *stdv, bf16 *__restrict__ x0)
 {
     chain_wait();
     chain_next();  // (after the wait, as above)
@@ -713,10 +712,9 @@ __global__ void k_output_compact(const float *__restrict__ y, int n3, int npts,
 // per thread: converting and adding every square in FP64 kept the narrow FP64
 // pipe busy for half of the kernel.
 constexpr int LOSS_PTS = 4;
-__global__ void __launch_bounds__(256) k_loss(const float *y, const float *__restrict__ xs,
-                                              const float *__restrict__ ts,
-                                              const float *__restrict__ sout, int nf, int n, int npts,
-                                              int B, float inv_count, bf16 *__restrict__ dy3,
+__global__ void __launch_bounds__(256) k_loss(const float *y, const float *xs, const float *ts,
+                                              const float *sout, int nf, int n, int npts, int B,
+                                              float inv_count, bf16 *__restrict__ dy3,
                                               double *__restrict__ part)
 {
     chain_wait();
