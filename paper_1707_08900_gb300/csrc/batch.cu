@@ -472,6 +472,7 @@ struct gbfd_batch {
     int cur;
     int zc;
     int kind;        // column routine (KIND_*)
+    bool kind_chosen;  // by the caller or the autotuner (else it follows the chunk length)
     int flow;        // 1: all substeps in one dataflow launch; 0: one launch per substep
     int stall_item;  // tests: a work item whose completion is never counted (-1 off)
     int grid;        // CTAs of a launch (0: resident CTAs of the kind on every SM)
@@ -557,6 +558,11 @@ gbfd_status build_items(gbfd_batch *b, int zc, int kind)
 // 32 planes, 15502 at 64; 8 x 64^3 597 -> 552 (16); 4 x 32^3 521 -> 195 (8).
 // With long columns of five fields the lagged routine is the faster one (96
 // boxes 15239), with short ones its longer start-up costs more.
+int default_kind(const gbfd_batch *b, int zc)
+{
+    return zc == 64 && b->nf == 5 ? KIND_LAG : KIND_PACKED;
+}
+
 void default_items(const gbfd_batch *b, int *zc, int *kind)
 {
     const double h = 3.0;
@@ -575,7 +581,7 @@ void default_items(const gbfd_batch *b, int *zc, int *kind)
             *zc = z;
         }
     }
-    *kind = *zc == 64 && b->nf == 5 ? KIND_LAG : KIND_PACKED;
+    *kind = default_kind(b, *zc);
 }
 
 int grid_of(const gbfd_batch *b) { return b->grid > 0 ? b->grid : b->grid_kind[b->kind]; }
@@ -815,6 +821,7 @@ gbfd_status gbfd_batch_init(int nbox, const int32_t *n, const double *lengths, c
     b->dflow = (Flow *)(b->ws + pl.off_flow);
     b->zc = 32;
     b->kind = KIND_PACKED;
+    b->kind_chosen = false;
     b->flow = 1;
     b->stall_item = -1;
     b->grid = 0;
@@ -1039,7 +1046,8 @@ gbfd_status gbfd_batch_set_option(gbfd_batch *b, int key, int64_t value)
     case GBFD_BATCH_OPT_ZCHUNK:
         if (value != 8 && value != 16 && value != 32 && value != 64)
             break;
-        return build_items(b, (int)value, b->kind);
+        return build_items(b, (int)value,
+                           b->kind_chosen ? b->kind : default_kind(b, (int)value));
     case GBFD_BATCH_OPT_GRID:
         if (value < 0 || value > 65535)
             break;
@@ -1049,6 +1057,7 @@ gbfd_status gbfd_batch_set_option(gbfd_batch *b, int key, int64_t value)
     case GBFD_BATCH_OPT_KERNEL:
         if (value < 0 || value >= NKIND)
             break;
+        b->kind_chosen = true;
         return build_items(b, b->zc, (int)value);
     case GBFD_BATCH_OPT_DATAFLOW:
         if (value != 0 && value != 1)
@@ -1155,6 +1164,7 @@ gbfd_status gbfd_batch_autotune(gbfd_batch *b, int steps, int *best_zc, double *
     if (e != cudaSuccess)
         return bcuda(b, e, "autotune");
     b->flow = bf;
+    b->kind_chosen = true;
     st = build_items(b, bz, bk);
     if (st != GBFD_OK)
         return st;
