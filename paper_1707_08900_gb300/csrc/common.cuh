@@ -250,8 +250,8 @@ struct FoldCubic {
 // by itself before the three are added.  In one sum with the common centre weight
 // VC the partial sums round against VC u until the last arm: at the viscous limit
 // of the time step (VC = 2.3) two FP32 steps were 2.1e-7 off (rms of the velocity at
-// 20^3 to 48^3) where the two-plane routine's separate second derivatives, which
-// these now are, leave 1.2e-7.
+// 20^3 to 48^3), with three sums 1.16e-7, the two-plane routine's unfolded
+// second derivatives 1.19e-7.
 struct FoldAxes {
     float l1[3], n1[3], v2[3], x2[3], cv, cx, m3[3];
     float nnu, nu23, ncs2, ns;
