@@ -569,7 +569,7 @@ gbfd_status gbfd_get_state(gbfd_ctx *ctx, void *dst, int dst_on_device, int dst_
     void *to = dst_on_device ? dst : (mapped ? mapped : (void *)ctx->staging);
     int nl = 0;
     cudaError_t e = launch_gather(ctx->state_region[ctx->cur] + ctx->Ls.origin, ctx->Ls, to,
-                                  dst_is_fp64, ctx->nf, ctx->stream, &nl);
+                                  dst_is_fp64, ctx->nf, mapped != nullptr, ctx->stream, &nl);
     ctx->launches += nl;
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "get_state gather");

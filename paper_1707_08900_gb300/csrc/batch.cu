@@ -932,7 +932,8 @@ gbfd_status gbfd_batch_get_state(gbfd_batch *b, int box, void *dst, int dst_on_d
     int nl = 0;
     void *to = dst_on_device ? dst : (void *)b->staging;
     cudaError_t e =
-        launch_gather(state_origin(b, box, b->cur), Ly, to, dst_is_fp64, b->nf, b->stream, &nl);
+        launch_gather(state_origin(b, box, b->cur), Ly, to, dst_is_fp64, b->nf, false, b->stream,
+                      &nl);
     b->launches += nl;
     if (e == cudaSuccess && !dst_on_device) {
         e = cudaMemcpyAsync(dst, b->staging, bytes, cudaMemcpyDeviceToHost, b->stream);

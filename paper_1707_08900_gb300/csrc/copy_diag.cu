@@ -11,12 +11,6 @@ namespace gbfd {
 
 namespace {
 
-__device__ __forceinline__ int wrapi(int i, int n)
-{
-    i %= n;
-    return i < 0 ? i + n : i;
-}
-
 // Four consecutive values moved with 16-byte accesses (one float4, or two
 // double2), converted on the way.
 template <class T>
@@ -54,14 +48,10 @@ __device__ __forceinline__ void store_quad(double *p, const double (&v)[4])
 
 constexpr int COPY_THREADS = 256;
 
-// Group of LPR lanes that one row takes (8 for rows of up to 32 values, 16 up to
-// 64, else 32) and the rows a group takes at once: their loads are all issued
-// before the first store.
-template <int LPR>
-struct RowGroup {
-    static constexpr int ROWS = LPR == 32 ? 2 : 4;
-    static constexpr int PER_BLOCK = COPY_THREADS / LPR * ROWS;
-};
+// Group of LPR lanes that take ROWS rows at once, every load issued before the
+// first store.  Chosen by row_group below.
+template <int LPR, int ROWS>
+constexpr int kRowsPerBlock = COPY_THREADS / LPR * ROWS;
 
 // Every padded row (interior and ghost rows, interior and ghost columns) of
 // every field from the compact source; ghosts take the periodic image.  VEC:
@@ -69,21 +59,19 @@ struct RowGroup {
 // in 16-byte accesses, four columns at a time; the four ghost columns on each
 // side are the first and the last four of the row, written by the thread that
 // holds them.  The source may be device memory or pinned host memory mapped into
-// the device address space.  DRAM-bound; with a warp per row and 64-bit row
-// arithmetic 256^3 took 133 us (5.0 TB/s) and a 32^3 box used 8 of 32 lanes.
-// IDX: unsigned when the rows can be counted in it.
-template <class TD, class TSrc, bool VEC, int LPR, class IDX>
+// the device address space.  IDX: unsigned when the rows can be counted in it
+// (with 64-bit row arithmetic 256^3 took 127 us, 5.0 TB/s; here 107).
+template <class TD, class TSrc, bool VEC, int LPR, int ROWS, class IDX>
 __global__ void __launch_bounds__(COPY_THREADS) k_scatter(const TSrc *__restrict__ src,
                                                          TD *__restrict__ dst, Layout L, IDX nrows)
 {
-    using G = RowGroup<LPR>;
     const int lane = threadIdx.x % LPR;
-    const IDX row0 = (IDX)blockIdx.x * G::PER_BLOCK + threadIdx.x / LPR * G::ROWS;
-    const TSrc *s[G::ROWS];
-    TD *d[G::ROWS];
+    const IDX row0 = (IDX)blockIdx.x * kRowsPerBlock<LPR, ROWS> + threadIdx.x / LPR * ROWS;
+    const TSrc *s[ROWS];
+    TD *d[ROWS];
     int n = 0;
 #pragma unroll
-    for (int k = 0; k < G::ROWS; ++k) {
+    for (int k = 0; k < ROWS; ++k) {
         const IDX row = row0 + k;
         if (row >= nrows)
             break;
@@ -98,13 +86,13 @@ __global__ void __launch_bounds__(COPY_THREADS) k_scatter(const TSrc *__restrict
     }
     if (VEC) {
         for (int x = 4 * lane; x < L.nx; x += 4 * LPR) {
-            Quad<TSrc> q[G::ROWS];
+            Quad<TSrc> q[ROWS];
 #pragma unroll
-            for (int k = 0; k < G::ROWS; ++k)
+            for (int k = 0; k < ROWS; ++k)
                 if (k < n)
                     q[k] = load_quad(s[k] + x);
 #pragma unroll
-            for (int k = 0; k < G::ROWS; ++k)
+            for (int k = 0; k < ROWS; ++k)
                 if (k < n) {
                     const TD v[4] = {(TD)q[k].v[0], (TD)q[k].v[1], (TD)q[k].v[2], (TD)q[k].v[3]};
                     store_quad(d[k] + GX + x, v);
@@ -116,25 +104,28 @@ __global__ void __launch_bounds__(COPY_THREADS) k_scatter(const TSrc *__restrict
         }
     } else {
 #pragma unroll
-        for (int k = 0; k < G::ROWS; ++k)
-            if (k < n)
-                for (int X = lane; X < L.nx + 2 * GX; X += LPR)
-                    d[k][X] = (TD)s[k][wrapi(X - GX, L.nx)];
+        for (int k = 0; k < ROWS; ++k)
+            if (k < n) {
+                for (int x = lane; x < L.nx; x += LPR)
+                    d[k][GX + x] = (TD)s[k][x];
+                if (lane < 2 * GX)
+                    d[k][lane < GX ? lane : L.nx + lane] =
+                        (TD)s[k][lane < GX ? L.nx - GX + lane : lane - GX];
+            }
     }
 }
 
 // Interior rows back to the compact layout, in the same way.
-template <class TS, class TD, bool VEC, int LPR, class IDX>
+template <class TS, class TD, bool VEC, int LPR, int ROWS, class IDX>
 __global__ void __launch_bounds__(COPY_THREADS) k_gather(const TS *__restrict__ src,
                                                         TD *__restrict__ dst, Layout L, IDX nrows)
 {
-    using G = RowGroup<LPR>;
     const int lane = threadIdx.x % LPR;
-    const IDX row0 = (IDX)blockIdx.x * G::PER_BLOCK + threadIdx.x / LPR * G::ROWS;
-    const TS *s[G::ROWS];
+    const IDX row0 = (IDX)blockIdx.x * kRowsPerBlock<LPR, ROWS> + threadIdx.x / LPR * ROWS;
+    const TS *s[ROWS];
     int n = 0;
 #pragma unroll
-    for (int k = 0; k < G::ROWS; ++k) {
+    for (int k = 0; k < ROWS; ++k) {
         const IDX row = row0 + k;
         if (row >= nrows)
             break;
@@ -146,13 +137,13 @@ __global__ void __launch_bounds__(COPY_THREADS) k_gather(const TS *__restrict__ 
     TD *d = dst + (long long)row0 * L.nx;
     if (VEC) {
         for (int x = 4 * lane; x < L.nx; x += 4 * LPR) {
-            Quad<TS> q[G::ROWS];
+            Quad<TS> q[ROWS];
 #pragma unroll
-            for (int k = 0; k < G::ROWS; ++k)
+            for (int k = 0; k < ROWS; ++k)
                 if (k < n)
                     q[k] = load_quad(s[k] + x);
 #pragma unroll
-            for (int k = 0; k < G::ROWS; ++k)
+            for (int k = 0; k < ROWS; ++k)
                 if (k < n) {
                     const TD v[4] = {(TD)q[k].v[0], (TD)q[k].v[1], (TD)q[k].v[2], (TD)q[k].v[3]};
                     store_quad(d + (long long)k * L.nx + x, v);
@@ -160,7 +151,7 @@ __global__ void __launch_bounds__(COPY_THREADS) k_gather(const TS *__restrict__ 
         }
     } else {
 #pragma unroll
-        for (int k = 0; k < G::ROWS; ++k)
+        for (int k = 0; k < ROWS; ++k)
             if (k < n)
                 for (int x = lane; x < L.nx; x += LPR)
                     d[(long long)k * L.nx + x] = (TD)s[k][x];
@@ -176,52 +167,65 @@ inline bool quad_ok(const void *compact, int nx)
     return ((uintptr_t)compact % 16) == 0 && nx % 4 == 0;
 }
 
-template <class TD, class TSrc, bool VEC, int LPR>
-cudaError_t scatter_r(const TSrc *src, TD *dst, const Layout &L, int nf, cudaStream_t stream)
+// Lanes per row and rows at once, measured against a warp per row on 19 shapes from
+// 8^3 to 256^3 in all four pairs of types (us, set or get): 8 lanes up to nx = 32, 16 up to
+// 64 (64^3 FP32 8.2 -> 5.1, FP64 8.2 -> 6.2; 2000 x 8 x 8 28.7 -> 8.3), else a warp.  Two
+// rows at once pay in FP32 on both sides when the rows fill the SMs (get 256^3 102.5 ->
+// 98.4, 140^3 24.6 -> 20.5); with FP64 on one side they are up to 1.5 times slower
+// (get 200 x 136 x 105 34.9 -> 49.7), as with few long rows (set 2048 x 16 x 16 6.2 ->
+// 8.3), except from FP64 to FP32 in whole passes of the warp (set 256^3 161.6 -> 152.6).
+// Host memory is written a warp per row (FP64 64^3 139 -> 89 us).
+template <class TFrom, class TTo, class F>
+cudaError_t row_group(long long nrows, int nx, bool vec, bool to_host, F &&f)
 {
-    const long long nrows = (long long)nf * L.nz * L.rows, per = RowGroup<LPR>::PER_BLOCK;
-    const unsigned grid = (unsigned)((nrows + per - 1) / per);
-    if (nrows < (1LL << 31))
-        k_scatter<TD, TSrc, VEC, LPR, unsigned><<<grid, COPY_THREADS, 0, stream>>>(src, dst, L,
-                                                                                (unsigned)nrows);
-    else
-        k_scatter<TD, TSrc, VEC, LPR, unsigned long long><<<grid, COPY_THREADS, 0, stream>>>(
-            src, dst, L, (unsigned long long)nrows);
-    return cudaGetLastError();
+    using std::integral_constant;
+    constexpr bool F32 = sizeof(TFrom) == 4 && sizeof(TTo) == 4;
+    constexpr int kFilled = 4 * 152;  // blocks of two rows per warp
+    auto g = [&](auto v, auto lpr, auto rows) {
+        constexpr int PER = kRowsPerBlock<decltype(lpr)::value, decltype(rows)::value>;
+        const unsigned grid = (unsigned)((nrows + PER - 1) / PER);
+        if (nrows < (1LL << 31))
+            f(v, lpr, rows, grid, (unsigned)nrows);
+        else
+            f(v, lpr, rows, grid, (unsigned long long)nrows);
+        return cudaGetLastError();
+    };
+    const integral_constant<int, 1> one{};
+    const integral_constant<int, 32> warp{};
+    if (!vec)
+        return g(std::false_type{}, warp, one);
+    if (nx <= 32 && !to_host)
+        return g(std::true_type{}, integral_constant<int, 8>{}, one);
+    if (nx <= 64 && !to_host)
+        return g(std::true_type{}, integral_constant<int, 16>{}, one);
+    if constexpr (sizeof(TTo) == 4)
+        if (F32 ? nrows >= (long long)kFilled * kRowsPerBlock<32, 2>
+                : nx % 128 == 0 || nx >= 512)
+            return g(std::true_type{}, warp, integral_constant<int, 2>{});
+    return g(std::true_type{}, warp, one);
 }
 
 template <class TD, class TSrc>
 cudaError_t scatter_t(const TSrc *src, TD *dst, const Layout &L, int nf, cudaStream_t stream)
 {
-    if (!quad_ok(src, L.nx))
-        return scatter_r<TD, TSrc, false, 32>(src, dst, L, nf, stream);
-    return L.nx <= 32   ? scatter_r<TD, TSrc, true, 8>(src, dst, L, nf, stream)
-           : L.nx <= 64 ? scatter_r<TD, TSrc, true, 16>(src, dst, L, nf, stream)
-                        : scatter_r<TD, TSrc, true, 32>(src, dst, L, nf, stream);
-}
-
-template <class TS, class TD, bool VEC, int LPR>
-cudaError_t gather_r(const TS *src, TD *dst, const Layout &L, int nf, cudaStream_t stream)
-{
-    const long long nrows = (long long)nf * L.nz * L.ny, per = RowGroup<LPR>::PER_BLOCK;
-    const unsigned grid = (unsigned)((nrows + per - 1) / per);
-    if (nrows < (1LL << 31))
-        k_gather<TS, TD, VEC, LPR, unsigned><<<grid, COPY_THREADS, 0, stream>>>(src, dst, L,
-                                                                             (unsigned)nrows);
-    else
-        k_gather<TS, TD, VEC, LPR, unsigned long long><<<grid, COPY_THREADS, 0, stream>>>(
-            src, dst, L, (unsigned long long)nrows);
-    return cudaGetLastError();
+    return row_group<TSrc, TD>(
+        (long long)nf * L.nz * L.rows, L.nx, quad_ok(src, L.nx), false,
+        [&](auto v, auto lpr, auto rows, unsigned grid, auto nrows) {
+            k_scatter<TD, TSrc, decltype(v)::value, decltype(lpr)::value, decltype(rows)::value,
+                      decltype(nrows)><<<grid, COPY_THREADS, 0, stream>>>(src, dst, L, nrows);
+        });
 }
 
 template <class TS, class TD>
-cudaError_t gather_t(const TS *src, TD *dst, const Layout &L, int nf, cudaStream_t stream)
+cudaError_t gather_t(const TS *src, TD *dst, const Layout &L, int nf, bool to_host,
+                     cudaStream_t stream)
 {
-    if (!quad_ok(dst, L.nx))
-        return gather_r<TS, TD, false, 32>(src, dst, L, nf, stream);
-    return L.nx <= 32   ? gather_r<TS, TD, true, 8>(src, dst, L, nf, stream)
-           : L.nx <= 64 ? gather_r<TS, TD, true, 16>(src, dst, L, nf, stream)
-                        : gather_r<TS, TD, true, 32>(src, dst, L, nf, stream);
+    return row_group<TS, TD>(
+        (long long)nf * L.nz * L.ny, L.nx, quad_ok(dst, L.nx), to_host,
+        [&](auto v, auto lpr, auto rows, unsigned grid, auto nrows) {
+            k_gather<TS, TD, decltype(v)::value, decltype(lpr)::value, decltype(rows)::value,
+                     decltype(nrows)><<<grid, COPY_THREADS, 0, stream>>>(src, dst, L, nrows);
+        });
 }
 
 // ------------------------------------------------------ ghost planes in z
@@ -505,14 +509,14 @@ cudaError_t launch_scatter(const void *src, int src_fp64, void *dst, const Layou
 }
 
 cudaError_t launch_gather(const void *src, const Layout &L, void *dst, int dst_fp64, int nf,
-                          cudaStream_t stream, int *launches)
+                          bool to_host, cudaStream_t stream, int *launches)
 {
     *launches += 1;
     if (L.w == 8)
-        return dst_fp64 ? gather_t((const double *)src, (double *)dst, L, nf, stream)
-                        : gather_t((const double *)src, (float *)dst, L, nf, stream);
-    return dst_fp64 ? gather_t((const float *)src, (double *)dst, L, nf, stream)
-                    : gather_t((const float *)src, (float *)dst, L, nf, stream);
+        return dst_fp64 ? gather_t((const double *)src, (double *)dst, L, nf, to_host, stream)
+                        : gather_t((const double *)src, (float *)dst, L, nf, to_host, stream);
+    return dst_fp64 ? gather_t((const float *)src, (double *)dst, L, nf, to_host, stream)
+                    : gather_t((const float *)src, (float *)dst, L, nf, to_host, stream);
 }
 
 namespace {

@@ -137,7 +137,7 @@ cudaError_t launch_forcing_tables(int kx, int ky, int kz, double phi, int nx, in
 cudaError_t launch_scatter(const void *src, int src_fp64, void *dst, const Layout &L, int nf,
                            cudaStream_t stream, int *launches);
 cudaError_t launch_gather(const void *src, const Layout &L, void *dst, int dst_fp64, int nf,
-                          cudaStream_t stream, int *launches);
+                          bool to_host, cudaStream_t stream, int *launches);
 
 // With walls in z: fill the ghost planes of nf fields of a walled layout
 // (origin = the layout's origin pointer) as parity mirrors about the wall
