@@ -890,7 +890,7 @@ __global__ void k_box_filter(const float *__restrict__ fine, Layout L, int nf, i
 // float-float (two_sum: every rounding error kept and added up, about 46
 // significant bits) because the FP64 pipe, with its conversions, bounds the
 // general kernel: (r + 1)^3 of both per value, 1022 us from 256^3 to 64^3, here
-// about 70 us (the fine state is 335 MB).  The weights and 1 / r^3 are powers of
+// 79 us (the fine state is 335 MB).  The weights and 1 / r^3 are powers of
 // two.  A sum that is not finite is formed again in FP64.
 template <int RR>
 __global__ void __launch_bounds__(256) k_box_filter_ff(const float *__restrict__ fine, Layout L,

@@ -89,8 +89,10 @@ cudaError_t launch_lag_shfl(const StateBufs &b, const Coef<float> &c, const RKSt
 // kernels taking turns find their code gone from the instruction caches, which
 // costs every launch 1 to 4 us.  Measured per substep, one kernel against three:
 // 32^3 4.2 and 5.1 us, 64^3 9.8 and 11.1, 96^3 19.2 and 21.5, 120 x 110 x 100
-// 35.3 and 39.7; 128^3 43.5 and 41.2, 200 x 136 x 105 52.6 and 48.6, 576 x 512 x
-// 452 8% in favour of three (160^3, one wave of CTAs, 71.1 and 74.7).
+// 35.3 and 39.7; 128^3 45.0 and 42.7, 200 x 136 x 105 57.1 and 51.5, 256^3 279 and 259.
+// Of 26 grids from 2^21 to 2^24 points three are faster on 23 (4 to 11%); the line
+// misses 160^3 (73.3 and 77.3), 160 x 157 x 159 (73.4 and 77.6) and 96 x 64 x 500 (59.4
+// and 64.3), for a reason that neither points nor waves of CTAs show.
 inline bool stage_kernels(const Layout &L)
 {
     return (long long)L.nx * L.ny * L.nz >= (1LL << 21);
