@@ -480,7 +480,9 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
             for (int k = (group + o0) & 1; k < m; k += EPI_GROUPS) {
                 const int o = o0 + k, z = z0 + k, slot = o % RING;
                 const long long p = (long long)b * n3 + ((long long)z * n + y) * n + x;
-                // the saved pre-activations, on their way during the wait
+                // the saved pre-activations, on their way during the wait (the
+                // forward pass wrote them several kernels ahead in the chain: read-only
+                // loads are safe)
                 float4 hv[EPI == EPI_DGELU ? NH / 4 : 1];
                 if constexpr (EPI == EPI_DGELU) {
                     if (inside)

@@ -260,8 +260,9 @@ def gbfd_diagnostics_noalloc(state_ptr, state_is_fp64, nx, ny, nz, nfields, lx, 
 
 
 def gbfd_autotune(ctx, reps=3, cache_path=None):
-    """Pick the fastest tile configuration (see include/gbfd.h); returns
-    (table index, ms per RK3 step, 0.0 on a cache hit)."""
+    """Pick the fastest of the built-in default and the tile table (see
+    include/gbfd.h); returns (table index, the one after the last for the
+    default, ms per RK3 step, 0.0 on a cache hit)."""
     cfg = ctypes.c_int()
     ms = ctypes.c_double()
     path = cache_path.encode() if cache_path else None
